@@ -120,7 +120,8 @@ typedef struct {
                               atoms per CTA, coalesced rows; large contexts).  Same
                               arithmetic, bit-identical results. */
     int list_lanes;        /* PAIR: lanes per bead-atom of the force kernel, 8, 16 or 32
-                              (0: 16).  Changes the summation order only. */
+                              (0: by the size of the context, 8 to 128).  Same results
+                              bit for bit; steps that may be recorded always use 16. */
     int rebuild_scope;     /* PAIR: 0 a list rebuild covers the systems one of whose
                               bead-atoms moved skin/2 (each system of a batch then runs
                               bit for bit as it would alone); 1 every system of the
@@ -303,7 +304,7 @@ int qtb_wait_selftest(qtb_ctx *c, int *gave_up, double *ms);
 typedef struct {
     double skin;          /* chosen neighbour-list skin, A (0: the default) */
     int nm_layout;        /* chosen ring-polymer integrator layout (1 compact, 2 wide; 0 if P = 1 only) */
-    int list_lanes;       /* chosen lanes per bead-atom of the force kernel (0: the default, 16) */
+    int list_lanes;       /* chosen lanes per bead-atom of the force kernel (0: the default) */
     int rebuild_scope;    /* chosen rebuild scope (0 requesting systems, 1 all; 0 for one system) */
     double ms_per_step;   /* mean device time of one MD step with that choice */
     double default_ms_per_step;  /* the same with the defaults (skin 0, nm_layout 0, list_lanes 0,
@@ -324,8 +325,8 @@ typedef struct {
  * configuration reached, its lists built on it, so that the timing sees the list
  * lengths and the rebuild rate of a long run rather than those of the initial
  * configuration (0: every candidate starts from the given positions).  The
- * candidates change the summation order and the rebuild schedule only, not the
- * dynamics.  Pair potentials only (QTB_ERR_ARG otherwise).  stream: as qtb_init.
+ * candidates change the summation order (through the skin) and the rebuild
+ * schedule only, not the dynamics.  Pair potentials only (QTB_ERR_ARG otherwise).  stream: as qtb_init.
  * Allocates and frees one context at a time; synchronises. */
 int qtb_autotune(const qtb_system *sys, int n_sys, const qtb_params *p, void *stream, int noise_mode, int n_taps,
                  double omega_max, int n_blocks, int equil_blocks, qtb_params *best, qtb_tuning *result);

@@ -69,7 +69,8 @@ struct qtb_ctx {
     std::vector<HSys> hs;
     std::vector<DSys> ds;
     std::vector<DRep> dr;
-    std::vector<int> cell_rep, icta_sys, lcta_rep, ccta_sys;
+    std::vector<int> cell_rep, icta_sys, ccta_sys;
+    std::vector<int2> units, units_rec;  // force units (Dev::units)
     Dev d{};
     MdLaunch ml{};
     PairTab tab{};
@@ -209,6 +210,58 @@ void fit_erfcx(double xmax, double c[12])
         for (int j = 0; j < n; ++j) Tm[k][j] = (j > 0 ? 2.0 * Tm[k - 1][j - 1] : 0.0) - Tm[k - 2][j];
     for (int k = 0; k < n; ++k)
         for (int j = 0; j < n; ++j) c[j] += a[k] * Tm[k][j];
+}
+
+// The damped Coulomb terms of the FP32 step kernel (pair_poly) as polynomials in
+// u = 2 r^2/rc^2 - 1: cf fits -al^3 (erf x - 2 x e^{-x^2}/sqrt(pi))/x^3 and ce fits
+// al erf(x)/x, x = al r (Chebyshev interpolation, converted to monomials).  False
+// when an error exceeds 1e-8 of 1/r^3 (cf) or 1/r (ce) at the cutoff: a sixth of an
+// FP32 rounding of the term they are taken from.
+bool fit_coulomb(double al, double rc, double *cf, double *ce)
+{
+    const int n = kFitN;
+    auto f = [&](int which, double r) {
+        const double x = al * r, x2 = x * x;
+        double s;
+        if (x < 0.5) {  // power series in x^2
+            double t = 1.0;
+            s = 0.0;
+            for (int k = 0; k < 16; ++k) {
+                s += t * (which ? 1.0 / (2 * k + 1) : 2.0 / (2 * k + 3));
+                t *= -x2 / (k + 1);
+            }
+            s *= 2.0 / std::sqrt(kPi);
+        } else {
+            s = which ? std::erf(x) / x : (std::erf(x) - 2.0 * x / std::sqrt(kPi) * std::exp(-x2)) / (x2 * x);
+        }
+        return which ? al * s : -al * al * al * s;
+    };
+    double Tm[kFitN][kFitN] = {{0}};
+    Tm[0][0] = 1.0;
+    Tm[1][1] = 1.0;
+    for (int k = 2; k < n; ++k)
+        for (int j = 0; j < n; ++j) Tm[k][j] = (j > 0 ? 2.0 * Tm[k - 1][j - 1] : 0.0) - Tm[k - 2][j];
+    bool ok = true;
+    for (int w = 0; w < 2; ++w) {
+        double *c = w ? ce : cf;
+        for (int k = 0; k < n; ++k) c[k] = 0.0;
+        for (int k = 0; k < n; ++k) {
+            double a = 0.0;
+            for (int i = 0; i < n; ++i) {
+                const double th = kPi * (i + 0.5) / n;
+                a += f(w, rc * std::sqrt(0.5 * (std::cos(th) + 1.0))) * std::cos(k * th);
+            }
+            a *= (k ? 2.0 : 1.0) / n;
+            for (int j = 0; j < n; ++j) c[j] += a * Tm[k][j];
+        }
+        for (int i = 0; i <= 400; ++i) {
+            const double u = -1.0 + i / 200.0, r = rc * std::sqrt(0.5 * (u + 1.0));
+            double p = 0.0;
+            for (int k = n - 1; k >= 0; --k) p = p * u + c[k];
+            if (!(std::fabs(p - f(w, r)) * (w ? rc : rc * rc * rc) <= 1e-8)) ok = false;
+        }
+    }
+    return ok;
 }
 
 static int decode_err_word(qtb_ctx *c, unsigned e);
@@ -712,6 +765,27 @@ double effective_skin(const qtb_params *p, double T)
     return p->skin < 0.0 ? 0.0 : p->skin;
 }
 
+// Lanes per bead-atom of the step kernel for a context of n bead-atoms (list_lanes
+// 0; the results do not depend on it).  A small context is bound by the chain of one
+// bead-atom's list rounds, so it takes more lanes while they still fit one wave of
+// CTAs; beyond a wave 16 lanes are the best compromise of instructions and occupancy,
+// but for the window where 8 lanes need one wave (6 CTAs per SM) and 16 two.  Measured
+// us per step on one GB300 (152 SMs; lanes 8 / 16 / 32 / 128): one-bead mixed form 216
+// ions 7.4 / 5.8 / 4.6 / 4.4, 512: 7.8 / 5.9 / 4.8 / 5.4, 4096: 8.9 / 9.3 / 8.0 / 19.3,
+// 8000: 15.1 / 10.7 / 14.7, 10648: 14.4 / 16.9 / 17.9, 32768: 36.9 / 32.0, 64000: 62.4 /
+// 62.8; ring polymers (7 CTAs per SM) 1728: 10.8 / 9.7 / 9.3, 4096: 13.9 / 13.4 / 14.9,
+// 55296: 76.4 / 70.7, 221184: 231 / 236, 864000: 887 / 917; FP64 form (bound by the
+// FP64 pipes, so its work is spread over the SMs) 64: 219 / 116 / 73 / 32, 512: 203 / 112 /
+// 83 / 61, 1728: 276 / 229 / 194 / 159, 4096: 630 / 369 / 385 / 364.
+int default_lanes(long long n, bool fp64, bool one_bead, int nsm)
+{
+    if (fp64) return n <= 27LL * nsm ? 128 : 16;
+    if (!one_bead) return n <= 14LL * nsm ? 32 : n <= 1024LL * nsm ? 16 : 8;
+    if (n <= 2LL * nsm) return 128;
+    if (n <= 28LL * nsm) return 32;                     // one wave: 7 CTAs of 4 bead-atoms per SM
+    return n > 56LL * nsm && n <= 96LL * nsm ? 8 : 16;  // 7 CTAs of 8; 6 CTAs of 16
+}
+
 int validate(const qtb_system *sys, int n_sys, const qtb_params *p)
 {
     if (!sys || n_sys < 1 || !p) return fail(QTB_ERR_ARG, "qtb_init: need n_sys >= 1 systems and params");
@@ -836,6 +910,7 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
                 T.eshift[t] = es;
             }
     }
+    bool poly_ok = false;  // the step kernel's polynomial Coulomb term is accurate enough
     {
         PairTabT<float> &F = c->tabf;
         memset(&F, 0, sizeof F);
@@ -861,6 +936,16 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
         double cfit[12];
         fit_erfcx(xmax, cfit);
         for (int k = 0; k < 12; ++k) F.erfc_c[k] = (float)cfit[k];
+        double cf[kFitN], ce[kFitN];
+        poly_ok = c->pair && T.alpha >= 0.0 && fit_coulomb(T.alpha, T.rc, cf, ce);
+        if (poly_ok) {
+            F.r2_us = (float)(2.0 / T.rc2);
+            for (int k = 0; k < kFitN; ++k) {
+                F.cf[k] = (float)cf[k];
+                F.ce[k] = (float)ce[k];
+            }
+        }
+        for (int t = 0; t < NT; ++t) F.nl2e_rho[t] = (float)(-log2e * T.inv_rho[t]);
     }
 
     // ---- layout
@@ -888,6 +973,14 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
     // cells (in the reference cell) and the lists keep that margin
     auto cell_edge_of = [&](int s) { return 0.5 * r_list_of(s) / (p->npt ? kCellMinScale : 1.0); };
     const double dens_margin = p->npt ? 1.0 / (kCellMinScale * kCellMinScale * kCellMinScale) : 1.0;
+    long long beads_total = 0;
+    for (int s = 0; s < n_sys; ++s) beads_total += (long long)sys[s].n_atoms * sys[s].n_beads;
+    int dev = 0, nsm = 0;
+    bool one_bead = true;
+    for (int s = 0; s < n_sys; ++s) one_bead = one_bead && sys[s].n_beads == 1;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return bail(fail(QTB_ERR_CUDA, "no CUDA device"));
+    const int lanes = p->list_lanes ? p->list_lanes : default_lanes(beads_total, !c->mixed, one_bead, nsm);
     int stage_cap = 0, maxnb = 32;
     if (c->pair) {
         double ecell = 0.0;
@@ -899,7 +992,8 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
             ecell = std::max(ecell, (double)sys[s].n_atoms / (nc[0] * nc[1] * nc[2]));
             // list capacity: 1.5 x the mean population of the list sphere plus a margin
             const double rho = sys[s].n_atoms / (sys[s].box[0] * sys[s].box[1] * sys[s].box[2]);
-            maxnb = std::max(maxnb, (int)roundup((long long)std::ceil(1.5 * rho * dens_margin * vlist + 64.0), 32));
+            maxnb = std::max(maxnb, (int)roundup((long long)std::ceil(1.5 * rho * dens_margin * vlist + 64.0),
+                                                 kColBlock));
         }
         // staging chunk of the list build: 1.5 x the mean stencil population plus a
         // margin, between 512 entries (the sort keys share the buffer) and 1024
@@ -910,13 +1004,10 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
     int nlcta = 0;
     // ring-polymer integrator layout: 32 atoms per CTA (coalesced rows) for large
     // contexts, fewer (more CTAs) for small ones
-    long long beads_total = 0;
-    for (int s = 0; s < n_sys; ++s) beads_total += (long long)sys[s].n_atoms * sys[s].n_beads;
     // bead-atom and dof indices are 32-bit on the device (3 dofs per bead-atom)
     if (beads_total > (long long)INT_MAX / 4)
         return bail(fail(QTB_ERR_ARG, "%lld bead-atoms in one context: at most %d", beads_total, INT_MAX / 4));
     const int nm_big = p->nm_layout == 2 ? 1 : p->nm_layout == 1 ? 0 : (beads_total >= (1LL << 18) ? 1 : 0);
-    const int lanes = p->list_lanes ? p->list_lanes : 16;
     for (int s = 0; s < n_sys; ++s) {
         const qtb_system &q = sys[s];
         HSys &h = c->hs[s];
@@ -998,11 +1089,12 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
                 R.cell0 = ncells;
                 ncells += cells;
                 R.fcta0 = nlcta;
-                const int nl = (h.N + list_atoms(lanes) - 1) / list_atoms(lanes);
-                nlcta += nl;
+                nlcta += (h.N + list_atoms(16) - 1) / list_atoms(16);
                 c->dr.push_back(R);
+                for (int a = 0; a < h.N; a += list_atoms(16)) c->units_rec.push_back(make_int2(nrep, a));
+                if (lanes != 16)
+                    for (int a = 0; a < h.N; a += list_atoms(lanes)) c->units.push_back(make_int2(nrep, a));
                 for (int t = 0; t < cells; ++t) c->cell_rep.push_back(nrep);
-                for (int t = 0; t < nl; ++t) c->lcta_rep.push_back(nrep);
                 ++nrep;
             }
             S.cell1 = ncells;
@@ -1018,11 +1110,11 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
     c->ml.lanes = lanes;
     // minimum image suffices for the list entries when every edge exceeds twice the
     // largest separation an entry can reach before a rebuild (r_cut + skin, plus skin/2
-    // of motion for each of the two atoms); not with a changing cell
-    c->ml.minimg = (c->pair && c->mixed && !p->npt) ? 1 : 0;
-    for (int s = 0; s < n_sys && c->ml.minimg; ++s)
+    // of motion for each of the two atoms); not with a changing cell.
+    c->ml.variant = (c->pair && c->mixed && poly_ok) ? (p->npt ? 1 : 2) : 0;
+    for (int s = 0; s < n_sys && c->ml.variant == 2; ++s)
         for (int k = 0; k < 3; ++k)
-            if (!(sys[s].box[k] > 2.0 * (p->r_cut + 2.0 * c->skins[s]))) c->ml.minimg = 0;
+            if (!(sys[s].box[k] > 2.0 * (p->r_cut + 2.0 * c->skins[s]))) c->ml.variant = 1;
     if (c->pair && step_prepare(c->ml, stage_cap) != cudaSuccess)
         return bail(fail(QTB_ERR_CUDA, "cannot prepare the cooperative step kernel (shared memory, occupancy)"));
     int ext_gx = 0;
@@ -1035,7 +1127,7 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
         if (c->pair) {
             // the system's replicas are consecutive, and so are their list force CTAs
             S.fcta0 = c->dr[S.rep0].fcta0;
-            S.fcta1 = c->dr[S.rep0 + c->hs[s].P - 1].fcta0 + (c->hs[s].N + list_atoms(lanes) - 1) / list_atoms(lanes);
+            S.fcta1 = c->dr[S.rep0 + c->hs[s].P - 1].fcta0 + (c->hs[s].N + list_atoms(16) - 1) / list_atoms(16);
             nforce = S.fcta1;
             S.grp0 = ngroups;
             S.ngrp = (S.fcta1 - S.fcta0 + kRedGroup - 1) / kRedGroup;
@@ -1053,8 +1145,10 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
     d.ncells = ncells;
     d.cap = cap;
     d.stage_cap = stage_cap;
-    d.nunits = nlcta;
+    d.nunits_rec = nlcta;
+    d.nunits = lanes == 16 ? nlcta : (int)c->units.size();
     d.maxnb = maxnb;
+    d.pshift = c->ml.variant == 2 ? 32 - kFixBits : 0;
     d.G = G;
     d.Dtot = D;
     d.obs_stride = p->obs_stride;
@@ -1131,7 +1225,8 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
     d.typ = upload(c, typ);
     d.rep = upload(c, c->dr);
     d.cell_rep = upload(c, c->cell_rep);
-    d.lcta_rep = upload(c, c->lcta_rep);
+    d.units_rec = upload(c, c->units_rec);
+    d.units = lanes == 16 ? d.units_rec : upload(c, c->units);
     d.icta_sys = upload(c, c->icta_sys);
     d.ccta_sys = ccta ? upload(c, c->ccta_sys) : nullptr;
     d.sys = upload(c, c->ds);
@@ -1148,21 +1243,14 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
         d.xref = c->alloc(psz * 3 * (size_t)G);
         d.nbr = (unsigned *)c->alloc(sizeof(unsigned) * (size_t)G * maxnb);
         d.nnb = (int *)c->alloc(sizeof(int) * (size_t)G);
-        if (!d.pos[0] || !d.pos[1] || !d.xref || !d.nbr || !d.nnb)
+        d.slot = (int *)c->alloc(sizeof(int) * (size_t)G);
+        d.cbase = (int *)c->alloc(sizeof(int) * (size_t)std::max(ncells, 1));
+        if (!d.pos[0] || !d.pos[1] || !d.xref || !d.nbr || !d.nnb || !d.slot || !d.cbase)
             return bail(fail(QTB_ERR_OOM, "neighbour-list allocation failed"));
-        // the type word of both packed position buffers (positions follow)
-        for (int k = 0; k < 2; ++k) {
-            if (c->mixed) {
-                std::vector<int4> pk((size_t)G);
-                for (size_t g = 0; g < (size_t)G; ++g) pk[g] = make_int4(0, 0, 0, typ[g]);
-                cudaMemcpyAsync(d.pos[k], pk.data(), sizeof(int4) * G, cudaMemcpyHostToDevice, c->st);
-            } else {
-                std::vector<double> pk(4 * (size_t)G, 0.0);
-                for (size_t g = 0; g < (size_t)G; ++g) pk[4 * g + 3] = (double)typ[g];
-                cudaMemcpyAsync(d.pos[k], pk.data(), sizeof(double) * 4 * G, cudaMemcpyHostToDevice, c->st);
-            }
-            if (cudaStreamSynchronize(c->st) != cudaSuccess) return bail(fail(QTB_ERR_CUDA, "upload failed"));
-        }
+        // the step kernel loads lists in whole blocks: words past a list's end are older
+        // entries or these zeros, valid slots either way
+        cudaMemsetAsync(d.nbr, 0, sizeof(unsigned) * (size_t)G * maxnb, c->st);
+        cudaMemsetAsync(d.slot, 0, sizeof(int) * (size_t)G, c->st);  // (a bead-atom that overflows its cell gets none)
         cudaMemsetAsync(d.nnb, 0, sizeof(int) * (size_t)G, c->st);
     }
     d.flag = (unsigned *)c->alloc(2 * sizeof(unsigned));

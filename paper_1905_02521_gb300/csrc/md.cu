@@ -455,8 +455,12 @@ __global__ void k_refresh_check(Dev d, int cur)
             }
             moved |= tot > lim;
             const int t = d.typ[g];
-            if (PM == PM_FIX) reinterpret_cast<int4 *>(d.pos[cur])[g] = make_int4((int)w[0], (int)w[1], (int)w[2], t);
-            else reinterpret_cast<D4 *>(d.pos[cur])[g] = D4{(double)w[0], (double)w[1], (double)w[2], (double)t};
+            const size_t sl = (size_t)S.g0 + (l / S.N) * S.N + d.slot[g];
+            if (PM == PM_FIX)
+                reinterpret_cast<int4 *>(d.pos[cur])[sl] = make_int4(pack_pos((int)w[0], d.pshift), pack_pos((int)w[1], d.pshift),
+                                                                     pack_pos((int)w[2], d.pshift), t);
+            else
+                reinterpret_cast<D4 *>(d.pos[cur])[sl] = D4{(double)w[0], (double)w[1], (double)w[2], (double)t};
         }
         if (moved) {
             atomicOr(&d.rflag[cur * d.nsys + s], 1u);
@@ -593,18 +597,21 @@ void launch_integrate(const Dev &d, const MdLaunch &m, int j, int cur, cudaStrea
 
 cudaError_t step_prepare(MdLaunch &m, int stage_entries)
 {
-    if (m.lanes == 8) return step_prepare_l8(m, stage_entries);
-    if (m.lanes == 32) return step_prepare_l32(m, stage_entries);
-    return step_prepare_l16(m, stage_entries);
+    cudaError_t e = step_prepare_l16(m, stage_entries);
+    if (e == cudaSuccess && m.lanes == 8) e = step_prepare_l8(m, stage_entries);
+    if (e == cudaSuccess && m.lanes == 32) e = step_prepare_l32(m, stage_entries);
+    if (e == cudaSuccess && m.lanes == 128) e = step_prepare_l128(m, stage_entries);
+    return e;
 }
 
 cudaError_t launch_force(const Dev &d, const MdLaunch &m, const PairTabT<float> &Tf, const PairTabT<double> &Td,
                          int kick, int j, int cur, int adv, int rec, cudaStream_t st)
 {
     if (m.pair) {
+        if (rec || m.lanes == 16) return step_force_l16(d, m, Tf, Td, kick, j, cur, adv, rec, st);
         if (m.lanes == 8) return step_force_l8(d, m, Tf, Td, kick, j, cur, adv, rec, st);
         if (m.lanes == 32) return step_force_l32(d, m, Tf, Td, kick, j, cur, adv, rec, st);
-        return step_force_l16(d, m, Tf, Td, kick, j, cur, adv, rec, st);
+        return step_force_l128(d, m, Tf, Td, kick, j, cur, adv, rec, st);
     }
     dim3 g((unsigned)m.n_ecta, (unsigned)d.nsys);
     if (m.mixed) k_force_ext<float><<<g, 128, 0, st>>>(d, Tf, kick);

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(128) k_integrate(Dev d, int j, int cur)
             X[o] = xn;
             if (PM != PM_FREE) {
                 const size_t g = S.g0 + (size_t)b * N + i;
-                reinterpret_cast<PS *>(d.pos[cur])[4 * g + c] = xn;
+                reinterpret_cast<PS *>(d.pos[cur])[4 * (g - i + d.slot[g]) + c] = pack_pos(xn, d.pshift);
                 const R dc = PosT<PM, R>::diff(xn, reinterpret_cast<const PS *>(d.xref)[o], fsc);
                 dd = dc * dc;
             }
@@ -506,12 +506,14 @@ __global__ void __launch_bounds__(nm_threads(P, BIG)) k_integrate_nm(Dev d, int 
                     tot = fma(dc, dc, tot);
                 }
                 moved |= tot > lim;
+                const size_t sl = gg - i + d.slot[gg];
                 if (PM == PM_FIX) {
                     int4 *pk = reinterpret_cast<int4 *>(d.pos[cur]);
-                    pk[gg] = make_int4((int)w3[0], (int)w3[1], (int)w3[2], tt[u]);
+                    pk[sl] = make_int4(pack_pos((int)w3[0], d.pshift), pack_pos((int)w3[1], d.pshift),
+                                       pack_pos((int)w3[2], d.pshift), tt[u]);
                 } else {
                     D4 *pk = reinterpret_cast<D4 *>(d.pos[cur]);
-                    pk[gg] = D4{(double)w3[0], (double)w3[1], (double)w3[2], (double)tt[u]};
+                    pk[sl] = D4{(double)w3[0], (double)w3[1], (double)w3[2], (double)tt[u]};
                 }
             }
         }

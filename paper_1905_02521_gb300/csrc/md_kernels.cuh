@@ -79,6 +79,11 @@ template <class R> struct PosT<PM_FREE, R> {  // unbounded (external potentials)
     __device__ static S wrap(S x, double) { return x; }
 };
 
+// a coordinate as the packed positions hold it (Dev::pos)
+__device__ __forceinline__ int pack_pos(int x, int shift) { return (int)((unsigned)x << shift); }
+__device__ __forceinline__ double pack_pos(double x, int) { return x; }
+__device__ __forceinline__ float pack_pos(float x, int) { return x; }
+
 __device__ __forceinline__ double warp_sum(double v)
 {
 #pragma unroll
@@ -121,18 +126,6 @@ struct FF {
             lo = __fadd_rn(__fadd_rn(lo, ol), e);
         }
     }
-    // sum over aligned groups of W lanes (W a power of two <= 32)
-    template <int W> __device__ void group_reduce()
-    {
-#pragma unroll
-        for (int o = W / 2; o > 0; o >>= 1) {
-            const float oh = __shfl_xor_sync(0xffffffffu, hi, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
-            float s, e;
-            two_sum(hi, oh, s, e);
-            hi = s;
-            lo = __fadd_rn(__fadd_rn(lo, ol), e);
-        }
-    }
     __device__ float value() const { return __fadd_rn(hi, lo); }
     // add another float-float value (bh + bl)
     __device__ void add_ff(float bh, float bl)
@@ -157,13 +150,42 @@ struct DD {
     double hi;
     __device__ void add(double x) { hi += x; }
     __device__ void warp_reduce() { hi = warp_sum(hi); }
-    template <int W> __device__ void group_reduce()
-    {
-#pragma unroll
-        for (int o = W / 2; o > 0; o >>= 1) hi += __shfl_xor_sync(0xffffffffu, hi, o);
-    }
     __device__ double value() const { return hi; }
 };
+
+// Sums of x, y and z over an aligned group of W lanes (8, 16 or 32), by halving: the
+// first exchange leaves a lane with x and y or with z, the second with one of them,
+// the rest add up that component.  Five float-float additions instead of twelve (the
+// reductions were a seventh of the step kernel's instructions at 16 lanes), each sum
+// over the same binary tree as a butterfly's.  Component c ends on the lanes
+// l = c W/4 .. c W/4 + W/4 - 1 (l: lane of the group); comp_of_lane(l) is c on the
+// first of them (it keeps the component's books), 3 elsewhere.
+template <int W> __device__ __forceinline__ int comp_of_lane(int l) { return (l & (W / 4 - 1)) ? 3 : l / (W / 4); }
+
+__device__ __forceinline__ void exchange_add(FF &keep, const FF &give, int o)
+{
+    keep.add_ff(__shfl_xor_sync(0xffffffffu, give.hi, o), __shfl_xor_sync(0xffffffffu, give.lo, o));
+}
+__device__ __forceinline__ void exchange_add(DD &keep, const DD &give, int o)
+{
+    keep.hi += __shfl_xor_sync(0xffffffffu, give.hi, o);
+}
+__device__ __forceinline__ void add_acc(FF &a, const FF &b) { a.add_ff(b.hi, b.lo); }
+__device__ __forceinline__ void add_acc(DD &a, const DD &b) { a.hi += b.hi; }
+template <int W, class ACC> __device__ __forceinline__ ACC reduce3(ACC x, ACC y, ACC z, int l)
+{
+    const bool h = (l & (W / 2)) != 0, q = (l & (W / 4)) != 0;
+    ACC zero{};
+    // lanes of the upper half keep z (and nothing), the lower ones x and y
+    ACC a = h ? z : x, b = h ? zero : y;
+    exchange_add(a, h ? x : z, W / 2);
+    exchange_add(b, h ? y : zero, W / 2);
+    ACC r = q ? b : a;
+    exchange_add(r, q ? a : b, W / 4);
+#pragma unroll
+    for (int o = W / 8; o > 0; o >>= 1) exchange_add(r, r, o);
+    return r;
+}
 
 template <int W, class T> __device__ __forceinline__ T group_sum(T v)
 {
@@ -189,8 +211,8 @@ static __device__ void cta_store_partials(const double *acc, double (*red)[kNQ],
 // FP32 form of the above for the list force kernel: the float-float sums of a
 // CTA's bead-atoms, stored as (hi, lo) pairs in out[0..kNQ).  The potential
 // energy and virial halves (en, w*) count on the lanes `lead` (one per
-// bead-atom), the kinetic energy kc + kl and momentum mc + ml of component c on
-// lane c of each LPA-lane group.  red is the CTA's [warps][kNQ] scratch (8 bytes
+// LPA-lane group of a warp), the kinetic energy kc + kl and momentum mc + ml of component c on
+// its lane of each LPA-lane group (comp_of_lane).  red is the CTA's [warps][kNQ] scratch (8 bytes
 // an entry).
 template <int LPA>
 static __device__ void cta_store_partials_ff(bool lead, float en, float w0, float w1, float w2, float w3, float w4,
@@ -213,9 +235,10 @@ static __device__ void cta_store_partials_ff(bool lead, float en, float w0, floa
     M.template across_groups<LPA>();
     // component c of the warp's kinetic energy goes to slot Q_K (c = 0) or to the
     // free slots 13 and 14, joined below
-    if (lane < 3) {
-        rf[warp][lane == 0 ? Q_K : 12 + lane] = make_float2(K.hi, K.lo);
-        rf[warp][Q_MOM + lane] = make_float2(M.hi, M.lo);
+    const int c = lane < LPA ? comp_of_lane<LPA>(lane) : 3;
+    if (c < 3) {
+        rf[warp][c == 0 ? Q_K : 12 + c] = make_float2(K.hi, K.lo);
+        rf[warp][Q_MOM + c] = make_float2(M.hi, M.lo);
     }
     if (lane == 0) rf[warp][Q_SPRING] = rf[warp][Q_X2] = rf[warp][15] = make_float2(0.f, 0.f);
     __syncthreads();
@@ -316,22 +339,21 @@ __device__ __forceinline__ void release_next_step() { asm volatile("griddepcontr
 // whose own request is set (rflag[cur]; every system with rebuild scope 1):
 // each system rebuilds on its own schedule, so that a system of a batch runs
 // exactly as it would alone.
-// bin_phase wraps the positions into the box (x, its packed copy pos[cur] and
-// the reference xref) and bins them into cells >= (r_cut + skin)/2 with atomic
-// slots; sort_phase puts each cell's slots in bead-atom order (so that every
-// list, and every later sum, has a fixed order); build_cell scans the 5^3
-// stencil of one cell.
+// bin_phase wraps the positions into the box (x and the reference xref) and bins
+// them into cells >= (r_cut + skin)/2 with atomic slots; sort_phase puts each
+// cell's slots in bead-atom order (so that every list, and every later sum, has a
+// fixed order) while scan_phase numbers the slots of a replica cell by cell;
+// build_cell gives the cell's bead-atoms their slots in the packed positions and
+// scans its 5^3 stencil.
 
 // one bead-atom g of replica R: wrap, pack, bin
 template <int PM>
-__device__ __forceinline__ void bin_one(const Dev &d, int cur, long long g, const DRep &R)
+__device__ __forceinline__ void bin_one(const Dev &d, long long g, const DRep &R)
 {
     typedef typename PosT<PM, double>::S PS;
-    typedef typename std::conditional<PM == PM_FIX, int4, D4>::type E4;
     const size_t G = (size_t)d.G;
     PS *X = reinterpret_cast<PS *>(d.x);
     PS *XR = reinterpret_cast<PS *>(d.xref);
-    PS w[3];
     int cc[3];
     for (int c = 0; c < 3; ++c) {
         const double L = R.box[c];
@@ -339,16 +361,11 @@ __device__ __forceinline__ void bin_one(const Dev &d, int cur, long long g, cons
         const PS xw = PosT<PM, double>::wrap(X[c * G + g], L);
         X[c * G + g] = xw;
         XR[c * G + g] = xw;
-        w[c] = xw;
         int v;
         if (PM == PM_FIX) v = (int)(((unsigned long long)(unsigned)xw * (unsigned)ncc) >> kFixBits);
         else v = (int)floor((double)xw / L * ncc);
         cc[c] = min(max(v, 0), ncc - 1);
     }
-    E4 p;
-    p.x = w[0]; p.y = w[1]; p.z = w[2];
-    if (PM == PM_FIX) p.w = d.typ[g]; else p.w = (double)d.typ[g];
-    reinterpret_cast<E4 *>(d.pos[cur])[g] = p;
     const int cell = R.cell0 + cc[0] + R.nc[0] * (cc[1] + R.nc[1] * cc[2]);
     const int slot = atomicAdd(&d.cnt[cell], 1);
     if (slot < d.cap)
@@ -371,11 +388,11 @@ __device__ void bin_phase(const Dev &d, int cur)
         // the grid-stride mapping of all bead-atoms, restricted to this system's range
         // (consecutive systems land on different threads)
         for (long long l = ((tid - S.g0) % nth + nth) % nth; l < gn; l += nth)
-            bin_one<PM>(d, cur, S.g0 + l, d.rep[S.rep0 + (int)(l / S.N)]);
+            bin_one<PM>(d, S.g0 + l, d.rep[S.rep0 + (int)(l / S.N)]);
     }
 }
 
-// one cell by one warp: slots in bead-atom order, packed positions
+// one cell by one warp: slots in bead-atom order, packed positions and types
 template <int PM>
 __device__ __forceinline__ void sort_cell(const Dev &d, int cell, int *kw, int lane)
 {
@@ -383,7 +400,6 @@ __device__ __forceinline__ void sort_cell(const Dev &d, int cell, int *kw, int l
     const int n = min(d.cnt[cell], d.cap);
     for (int e = lane; e < n; e += 32) kw[e] = d.cidx[(size_t)cell * d.cap + e];
     __syncwarp();
-    const int g0 = d.rep[d.cell_rep[cell]].g0;
     for (int e = lane; e < n; e += 32) {
         const int g = kw[e];
         int rank = 0;
@@ -392,16 +408,46 @@ __device__ __forceinline__ void sort_cell(const Dev &d, int cell, int *kw, int l
         d.cidx[o] = g;
         if (PM == PM_FIX) {
             const int *X = reinterpret_cast<const int *>(d.x);
-            reinterpret_cast<int4 *>(d.cpos)[o] = make_int4(X[g], X[G + g], X[2 * G + g], g - g0);
+            reinterpret_cast<int4 *>(d.cpos)[o] = make_int4(X[g], X[G + g], X[2 * G + g], d.typ[g]);
         } else {
             const double *X = reinterpret_cast<const double *>(d.x);
-            reinterpret_cast<D4 *>(d.cpos)[o] = D4{X[g], X[G + g], X[2 * G + g], (double)(g - g0)};
+            reinterpret_cast<D4 *>(d.cpos)[o] = D4{X[g], X[G + g], X[2 * G + g], (double)d.typ[g]};
         }
     }
     __syncwarp();
-    if (lane == 0) {
-        d.ccount[cell] = n;
-        d.cnt[cell] = 0;
+    if (lane == 0) d.ccount[cell] = n;
+}
+
+// first slot of every cell of the requesting systems' replicas: an exclusive scan
+// of the cell counts, one CTA per replica (from the end of the grid, beside the
+// sorting of the first CTAs); each thread scans a run of consecutive cells
+static __device__ void scan_phase(const Dev &d, int cur, int *warp_sums)
+{
+    const unsigned *rf = d.rflag + cur * d.nsys;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int r = (int)(gridDim.x - 1 - blockIdx.x); r < d.nrep; r += gridDim.x) {
+        const DRep &R = d.rep[r];
+        if (!d.rebuild_all && rf[R.sys] == 0u) continue;  // uniform over the CTA
+        const int nc = R.nc[0] * R.nc[1] * R.nc[2], per = (nc + (int)blockDim.x - 1) / (int)blockDim.x;
+        const int c0 = R.cell0 + min(nc, (int)threadIdx.x * per), c1 = R.cell0 + min(nc, ((int)threadIdx.x + 1) * per);
+        int run = 0;
+        for (int c = c0; c < c1; ++c) run += min(d.cnt[c], d.cap);
+        int incl = run;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        __syncthreads();
+        if (lane == 31) warp_sums[warp] = incl;
+        __syncthreads();
+        int base = incl - run;
+        for (int w = 0; w < nw; ++w)
+            if (w < warp) base += warp_sums[w];
+        for (int c = c0; c < c1; ++c) {
+            d.cbase[c] = base;
+            base += min(d.cnt[c], d.cap);
+        }
     }
 }
 
@@ -423,7 +469,7 @@ __device__ void sort_phase(const Dev &d, int cur, int *keys)
 
 // List build.  One CTA per home cell: its warps stage the stencil cells
 // (sorted slots; image shift added, fixed point + m 2^30 in wrapping int32
-// arithmetic; entry word = local index | image bits) chunk by chunk, and for
+// arithmetic; the list entry, see kNbIdx, in the last word) chunk by chunk, and for
 // each chunk every warp takes one home bead-atom at a time, scans the flat
 // staged array and appends the entries within r_cut + skin to the bead-atom's
 // list, so that a list is in stencil scan order.
@@ -432,12 +478,12 @@ constexpr int kStencil = (2 * kStencilHalf + 1) * (2 * kStencilHalf + 1) * (2 * 
 
 // shared memory of build_cell (besides the staging chunk)
 struct BuildSmem {
-    int soff[kStencil + 1], scell[kStencil], simg[kStencil][3];
+    int soff[kStencil + 1], scell[kStencil], sbase[kStencil], simg[kStencil][3];
     int scount[kMaxCellCap];
 };
 
 template <int PM, class R>
-__device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, void *stage_mem, BuildSmem &B)
+__device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, int cur, void *stage_mem, BuildSmem &B)
 {
     typedef typename std::conditional<PM == PM_FIX, int4, D4>::type E4;
     constexpr int SH = kStencilHalf, SW = 2 * kStencilHalf + 1;
@@ -450,6 +496,18 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, void *stage_mem
     if (cnt == 0) return;  // uniform over the CTA
     const DRep RP = d.rep[d.cell_rep[cell]];
     const int lc = cell - RP.cell0;
+    if (threadIdx.x == 0) d.cnt[cell] = 0;  // for the next rebuild's binning (the scan has read it)
+    // the cell's bead-atoms: their slots, and the packed positions there (the other
+    // buffer gets the types: the one-bead step writes only coordinates to it)
+    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+        const size_t o = (size_t)cell * d.cap + t;
+        const int sl = d.cbase[cell] + t;
+        E4 p = reinterpret_cast<const E4 *>(d.cpos)[o];
+        p.x = pack_pos(p.x, d.pshift); p.y = pack_pos(p.y, d.pshift); p.z = pack_pos(p.z, d.pshift);
+        d.slot[d.cidx[o]] = sl;
+        reinterpret_cast<E4 *>(d.pos[cur])[(size_t)RP.g0 + sl] = p;
+        reinterpret_cast<E4 *>(d.pos[cur ^ 1])[(size_t)RP.g0 + sl].w = p.w;
+    }
     const int cx = lc % RP.nc[0], cy = (lc / RP.nc[0]) % RP.nc[1], cz = lc / (RP.nc[0] * RP.nc[1]);
     for (int t = threadIdx.x; t < kStencil; t += blockDim.x) {
         const int ox = t % SW - SH, oy = (t / SW) % SW - SH, oz = t / (SW * SW) - SH;
@@ -458,6 +516,7 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, void *stage_mem
         ux -= mx * RP.nc[0]; uy -= my * RP.nc[1]; uz -= mz * RP.nc[2];
         const int nc = RP.cell0 + ux + RP.nc[0] * (uy + RP.nc[1] * uz);
         scell[t] = nc;
+        B.sbase[t] = d.cbase[nc];
         simg[t][0] = mx; simg[t][1] = my; simg[t][2] = mz;
         soff[t + 1] = d.ccount[nc];
     }
@@ -508,12 +567,12 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, void *stage_mem
         constexpr int U = 4;
         for (int base = 0; base < cn; base += U * (int)blockDim.x) {
             E4 buf[U];
-            int tcell[U], dst[U];
+            int tcell[U], dst[U], rank[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int el = base + u * (int)blockDim.x + (int)threadIdx.x;
                 dst[u] = -1;
-                tcell[u] = 0;
+                tcell[u] = rank[u] = 0;
                 if (el < cn) {
                     const int e = c0 + el;
                     int lo = 0, hi = kStencil - 1;  // stencil cell t with soff[t] <= e < soff[t+1]
@@ -523,6 +582,7 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, void *stage_mem
                     }
                     tcell[u] = lo;
                     dst[u] = el;
+                    rank[u] = e - soff[lo];
                     buf[u] = reinterpret_cast<const E4 *>(d.cpos)[(size_t)scell[lo] * d.cap + (e - soff[lo])];
                 }
             }
@@ -533,16 +593,18 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, void *stage_mem
                 const int t = tcell[u];
                 const int mx = simg[t][0], my = simg[t][1], mz = simg[t][2];
                 const unsigned ib = ((unsigned)(mx & 3) << 26) | ((unsigned)(my & 3) << 28) | ((unsigned)(mz & 3) << 30);
+                const unsigned sl = (unsigned)(B.sbase[t] + rank[u]);
+                const unsigned ent = (PM == PM_FIX && d.pshift) ? sl << 4 : sl | ib;
                 if (PM == PM_FIX) {
                     p.x = (int)((unsigned)p.x + (unsigned)mx * (1u << kFixBits));
                     p.y = (int)((unsigned)p.y + (unsigned)my * (1u << kFixBits));
                     p.z = (int)((unsigned)p.z + (unsigned)mz * (1u << kFixBits));
-                    p.w = (int)((unsigned)p.w | ib);
+                    p.w = (int)ent;
                 } else {
                     p.x += mx * RP.box[0];
                     p.y += my * RP.box[1];
                     p.z += mz * RP.box[2];
-                    p.w = (double)((unsigned)p.w | ib);
+                    p.w = (double)ent;
                 }
                 stage[dst[u]] = p;
             }
@@ -576,7 +638,8 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, void *stage_mem
                 const unsigned m = __ballot_sync(0xffffffffu, take);
                 if (take) {
                     const int k = n + __popc(m & lt);
-                    if (k < maxnb) row[k] = (unsigned)pj.w;
+                    // (blocks in the order of the step kernel's loads, see kCols)
+                    if (k < maxnb) row[(k & ~(kColBlock - 1)) + (k & (kCols - 1)) * kColNE + (k / kCols) % kColNE] = (unsigned)pj.w;
                 }
                 n += __popc(m);
             };
@@ -613,10 +676,11 @@ template <class R> struct alignas(8 * sizeof(R)) PairRow {
     R inv_rho, A_over_rho, C6, qq, A, C, eshift, pad;
 };
 
-template <class R> __device__ __forceinline__ PairRow<R> pair_row(const PairTabT<R> &T, int t)
+template <int VAR, class R> __device__ __forceinline__ PairRow<R> pair_row(const PairTabT<R> &T, int t)
 {
     PairRow<R> p;
-    p.inv_rho = T.inv_rho[t]; p.A_over_rho = T.A_over_rho[t]; p.C6 = T.C6[t]; p.qq = T.qq[t];
+    p.inv_rho = VAR ? T.nl2e_rho[t] : T.inv_rho[t];  // (pair_poly takes the exponent in units of ln 2)
+    p.A_over_rho = T.A_over_rho[t]; p.C6 = T.C6[t]; p.qq = T.qq[t];
     p.A = T.A[t]; p.C = T.C[t]; p.eshift = T.eshift[t]; p.pad = R(0);
     return p;
 }
@@ -650,6 +714,59 @@ __device__ __forceinline__ void pair_eval(const PairTabT<float> &T, const PairRo
     if (energy) {
         const float ec = fmaf(er, rinv, fmaf(T.fshift, r - T.rc, -T.erfc_rc_over_rc));
         e = fmaf(qq, ec, fmaf(P2.A, ex, fmaf(-P2.C, r6i, -P2.eshift)));
+    } else {
+        e = 0.0f;
+    }
+}
+
+__device__ __forceinline__ float ex2_ftz(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rsqrt_ftz(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// The same, FP32 form, variants 1 and 2 of the step kernel: since
+//   erfc(x)/r^2 + 2 alpha e^{-x^2}/(sqrt(pi) r) = 1/r^2 - r alpha^3 t(x^2),
+//   t = (erf x - 2 x e^{-x^2}/sqrt(pi))/x^3  (entire in x^2, x = alpha r),
+// the damped Coulomb force over r is qq (r^-3 - fshift/r - alpha^3 t), one
+// polynomial in r^2 with no exponential; alpha erf(x)/x, entire too, gives the
+// energy.  The step kernel is bound by its instructions (issue slots 72 % busy on
+// 64000 ions), so this form matters: with 1/r and 1/r^2 from one Newton step each,
+// e^{-r/rho} as 2^a (1 + err(a) ln 2), a = -r log2(e)/rho and err(a) its exact
+// rounding error, a pair takes ~32 instructions instead of ~50, and fewer of its
+// roundings are at the size of 1/r^3: its force error against 64 bits is smaller than
+// that of the form above (modelled: 6.5e-6 against 8.0e-6 relative L2 on 512-ion MgO,
+// 5.8e-6 against 7.4e-6 on LiH).  The context takes it when the fits are accurate to
+// 1e-8 of the Coulomb term at the cutoff (alpha r_cut up to ~1.75).
+__device__ __forceinline__ void pair_poly(const PairTabT<float> &T, const PairRow<float> &P2, float r2, float &f_over_r,
+                                          float &e, bool energy)
+{
+    const float y = rsqrt_ftz(r2), t = y * y;
+    const float rinv = y * fmaf(-0.5f * r2, t, 1.5f), r2i = fmaf(t, fmaf(-r2, t, 1.0f), t);
+    const float r = r2 * rinv;
+    const float r4i = r2i * r2i, r8i = r4i * r4i;
+    const float u = fmaf(r2, T.r2_us, -1.0f);
+    float p = T.cf[kFitN - 1];
+#pragma unroll
+    for (int k = kFitN - 2; k >= 0; --k) p = fmaf(p, u, T.cf[k]);
+    p = fmaf(r2i, rinv, fmaf(-T.fshift, rinv, p));  // one rounding at the size of 1/r^3
+    const float a = r * P2.inv_rho;
+    float ex = ex2_ftz(a);
+    ex = fmaf(ex * 0.69314718f, fmaf(r, P2.inv_rho, -a), ex);
+    f_over_r = fmaf(P2.qq, p, fmaf(P2.A_over_rho * ex, rinv, -(P2.C6 * r8i)));
+    if (energy) {
+        float q = T.ce[kFitN - 1];
+#pragma unroll
+        for (int k = kFitN - 2; k >= 0; --k) q = fmaf(q, u, T.ce[k]);
+        const float ec = (rinv - q) + fmaf(T.fshift, r - T.rc, -T.erfc_rc_over_rc);
+        e = fmaf(P2.qq, ec, fmaf(P2.A, ex, fmaf(-P2.C, r4i * r2i, -P2.eshift)));
     } else {
         e = 0.0f;
     }
@@ -897,18 +1014,18 @@ __device__ void cell_update(const Dev &d, int s, long long n, int cur)
 }
 
 // ---------------------------------------------------------------------------
-// Pair force from the neighbour lists: LPA lanes per home bead-atom
-// (32 / LPA bead-atoms per warp), each lane strides through the list with two
-// independent entries per iteration and the next iteration's entries already
-// requested; every entry is evaluated and masked by r < r_cut (no divergent
-// branch).  Epilogue on the first three lanes of a group (one Cartesian
+// Pair force from the neighbour lists: LPA lanes per home bead-atom (8 or 16: several
+// bead-atoms per warp; 128: a CTA each), each lane takes the kColNE entries of one
+// column of a list block at a time, with one load, the next ones already requested;
+// every entry is evaluated and masked by r < r_cut (no divergent branch).  Epilogue
+// on three lanes of a bead-atom (one Cartesian
 // component each): force (times 1/P, Eq. 4), the closing B(dt/2) kick, the
 // observables of recorded steps and, with ADV (one-bead systems), the first
 // half of the next step: B(dt/2), A(dt/2) O(dt) A(dt/2) with the next step's
 // coloured noise, written to x and pos[cur ^ 1], and the rebuild test for the
 // next step.  Recorded steps: the last CTA of a system reduces its partials.
 
-template <int PM, class R, int ADV, int REC, int LPA, int MI>
+template <int PM, class R, int ADV, int REC, int LPA, int VAR>
 __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, const PairRow<R> *ptab, int kick,
                                            int j, int cur, int u, double (*red)[kNQ], double (*rsh)[kNQ + 1],
                                            int &s_last)
@@ -916,11 +1033,14 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
     typedef typename std::conditional<PM == PM_FIX, int4, D4>::type E4;
     typedef typename std::conditional<sizeof(R) == 4, FF, DD>::type ACC;
     typedef typename PosT<PM, R>::S PS;
-    constexpr int APW = 32 / LPA;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int sub = lane & (LPA - 1), grp = lane / LPA;
-    const DRep RP = d.rep[d.lcta_rep[u]];
-    const int i = (u - RP.fcta0) * list_atoms(LPA) + warp * APW + grp;
+    static_assert(LPA == 8 || LPA == 16 || LPA == 32 || LPA == 128, "lanes per bead-atom");
+    static_assert(!REC || LPA == 16, "the recording variants have 16 lanes");
+    constexpr int LW = LPA < 16 ? LPA : 16;  // lanes that share the reduction and the epilogue
+    constexpr bool MI = VAR == 2;
+    const int lane = threadIdx.x & 31, sub = threadIdx.x & (LPA - 1);
+    const int2 unit = (REC ? d.units_rec : d.units)[u];
+    const DRep RP = d.rep[unit.x];
+    const int i = unit.y + (int)threadIdx.x / LPA;
     const bool act = i < RP.N;
     const long long step = d.clock[0] * kBlockSteps + j + 1;
     // (isothermal-isobaric runs reduce K and the virial every step: the cell needs them)
@@ -928,20 +1048,20 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
     const DSys &S = d.sys[RP.sys];
     const size_t G = (size_t)d.G;
     const long long gi = RP.g0 + (act ? i : 0);
-    const E4 *Pc = reinterpret_cast<const E4 *>(d.pos[cur]);
-    const E4 *Pr = Pc + RP.g0;
-    const E4 hp = Pc[gi];
+    const E4 *Pr = reinterpret_cast<const E4 *>(d.pos[cur]) + RP.g0;
+    const int sl = d.slot[gi];
+    const E4 hp = Pr[sl];
     int ti;
     if (PM == PM_FIX) ti = hp.w; else ti = (int)hp.w;
     const int n = act ? min(d.nnb[gi], d.maxnb) : 0;
-    const unsigned *row = d.nbr + (size_t)gi * d.maxnb;
+    const uint4 *row = reinterpret_cast<const uint4 *>(d.nbr + (size_t)gi * d.maxnb);
     // physical distances: the reference cell's, scaled by lam in an isothermal-isobaric run
     // (such runs launch the recording variants only: the others carry no cell code)
     const DNpt *NC = (REC && d.npt && d.npt[RP.sys].on) ? d.npt + RP.sys : nullptr;
     const R lam = NC ? (sizeof(R) == 4 ? (R)NC->lamf : (R)NC->lam) : R(1);
     const R sx = (R)RP.fix_scale[0] * lam, sy = (R)RP.fix_scale[1] * lam, sz = (R)RP.fix_scale[2] * lam;
     const R rc2 = T.rc2;
-    ACC fx{}, fy{}, fz{};
+    ACC fx{}, fy{}, fz{}, f1x{}, f1y{}, f1z{};  // (f1: the second column of a lane, 8 lanes)
     R en = 0, w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0, w5 = 0;
     struct Geo {
         R dx, dy, dz, r2;
@@ -949,18 +1069,18 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
     };
     // r_j + image - r_i of one list entry
     auto geo = [&](unsigned e) {
-        const E4 pj = Pr[e & kNbIdx];
+        const E4 pj = MI ? *reinterpret_cast<const E4 *>(reinterpret_cast<const char *>(Pr) + e) : Pr[e & kNbIdx];
         Geo g;
         if (PM == PM_FIX) {
             // exact in wrapping 32-bit arithmetic
             if constexpr (MI) {
                 // MI: every cell exceeds twice the largest separation a list entry can
-                // reach, so the difference modulo the 30-bit edge, sign-extended, is the
-                // entry's image (4 x the difference, exact in float, times scale/4: the
-                // same value as below, without decoding the image bits)
-                g.dx = (R)(int)(((unsigned)pj.x - (unsigned)hp.x) << 2) * (sx * R(0.25));
-                g.dy = (R)(int)(((unsigned)pj.y - (unsigned)hp.y) << 2) * (sy * R(0.25));
-                g.dz = (R)(int)(((unsigned)pj.z - (unsigned)hp.z) << 2) * (sz * R(0.25));
+                // reach, so the difference modulo the edge, sign-extended, is the entry's
+                // image (positions shifted to 32 bits: 4 x the difference, exact in float,
+                // times scale/4: the same value as below, without decoding the image bits)
+                g.dx = (R)(int)((unsigned)pj.x - (unsigned)hp.x) * (sx * R(0.25));
+                g.dy = (R)(int)((unsigned)pj.y - (unsigned)hp.y) * (sy * R(0.25));
+                g.dz = (R)(int)((unsigned)pj.z - (unsigned)hp.z) * (sz * R(0.25));
             } else {
                 g.dx = (R)(int)((unsigned)pj.x + ((e << 4) & 0xC0000000u) - (unsigned)hp.x) * sx;
                 g.dy = (R)(int)((unsigned)pj.y + ((e << 2) & 0xC0000000u) - (unsigned)hp.y) * sy;
@@ -988,7 +1108,8 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
     // added to the round's partial sums (px, py, pz)
     auto force = [&](const Geo &g, bool in, R &px, R &py, R &pz) {
         R fo, ee;
-        pair_eval(T, ptab[ti * kMaxTypes + g.tj], g.r2, fo, ee, REC && rec);
+        if constexpr (VAR) pair_poly(T, ptab[ti * kMaxTypes + g.tj], g.r2, fo, ee, REC && rec);
+        else pair_eval(T, ptab[ti * kMaxTypes + g.tj], g.r2, fo, ee, REC && rec);
         fo = in ? fo : R(0);
         // stored displacement is r_j - r_i: the force on i is -fo (r_j - r_i)
         px = fma(-fo, g.dx, px); py = fma(-fo, g.dy, py); pz = fma(-fo, g.dz, pz);
@@ -998,48 +1119,113 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
             w3 = fma(fo * g.dx, g.dy, w3); w4 = fma(fo * g.dx, g.dz, w4); w5 = fma(fo * g.dy, g.dz, w5);
         }
     };
+    // One column of a block (kColNE entries) is a group: its terms are summed in R, the
+    // groups' sums then added up error-free (float-float; FP64 form: in FP64) column by
+    // column in block order, the columns at last over a binary tree.  So the sums are
+    // the same whatever the lane count: 16 lanes take a column each; 8 two; 32 and 128
+    // take two and eight blocks at a time and hand the groups' sums to the lanes that
+    // add them up.  (The extra roundings of a group are those of kColNE - 1 additions
+    // of terms of like size: no change of the error budget, modelled on the CPU.)
+    // A group's entries are loaded while the one before is evaluated (blocks past the
+    // list's end: entry 0, masked; words past its end inside a block hold older
+    // entries, valid slots, masked too).  The lists end with the skin-shell entries: a
+    // group in which no lane of the warp has an entry within r_cut skips the pair terms
+    // (they would add exact zeros).
     {
-        // entries k + q LPA (q < NE) of this lane; the next NE are requested before
-        // the current ones are evaluated (slots past the end read entry 0, masked).
-        // The lists end with the skin-shell entries: a round in which no lane of
-        // the warp has an entry within r_cut skips the pair terms (they would add
-        // exact zeros).  The trip count is the warp's longest list, so the vote
-        // is uniform.
-        constexpr int NE = 4;
-        int nmax = n;
+        const int nblk = (n + kColBlock - 1) / kColBlock;
+        auto entries = [&](int b, int v) { return b < nblk ? row[b * kCols + v] : make_uint4(0u, 0u, 0u, 0u); };
+        // the sums of the group's terms go to `sink` (unless every lane's are zero)
+        auto group = [&](const uint4 &e4, int b, int v, auto sink) {
+            const unsigned e[kColNE] = {e4.x, e4.y, e4.z, e4.w};
+            const int left = n - v - b * kColBlock;  // entries from the column's first one on
+            Geo g[kColNE];
+            bool in[kColNE], any = false;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
-        unsigned e[NE];
+            for (int q = 0; q < kColNE; ++q) g[q] = geo(e[q]);
 #pragma unroll
-        for (int q = 0; q < NE; ++q) e[q] = (sub + q * LPA < n) ? row[sub + q * LPA] : 0u;
-        for (int k0 = 0; k0 < nmax; k0 += NE * LPA) {
-            const int k = k0 + sub, kn = k + NE * LPA;
-            unsigned e2[NE];
-#pragma unroll
-            for (int q = 0; q < NE; ++q) e2[q] = (kn + q * LPA < n) ? row[kn + q * LPA] : 0u;
-            Geo g[NE];
-            bool in[NE], any = false;
-#pragma unroll
-            for (int q = 0; q < NE; ++q) {
-                g[q] = geo(e[q]);
-                in[q] = (k + q * LPA < n) && (g[q].r2 < rc2);
+            for (int q = 0; q < kColNE; ++q) {
+                in[q] = (q * kCols < left) && (g[q].r2 < rc2);
                 any |= in[q];
             }
             if (__any_sync(0xffffffffu, any)) {
-                // the round's NE terms are summed in R, the partial sum then added
-                // error-free (float-float): the extra roundings are those of NE - 1
-                // additions of terms of like size (modelled on the CPU: no change of
-                // the error budget)
                 R px = 0, py = 0, pz = 0;
 #pragma unroll
-                for (int q = 0; q < NE; ++q) force(g[q], in[q], px, py, pz);
-                fx.add(px); fy.add(py); fz.add(pz);
+                for (int q = 0; q < kColNE; ++q) force(g[q], in[q], px, py, pz);
+                sink(px, py, pz);
             }
+        };
+        auto add0 = [&](R px, R py, R pz) { fx.add(px); fy.add(py); fz.add(pz); };
+        if constexpr (LPA <= 16) {
+            // the trip count is the warp's longest list, so the votes are uniform
+            int bmax = nblk;
 #pragma unroll
-            for (int q = 0; q < NE; ++q) e[q] = e2[q];
+            for (int o = 16; o >= LPA; o >>= 1) bmax = max(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
+            uint4 ea = entries(0, sub);
+            if constexpr (LPA == 8) {
+                for (int b = 0; b < bmax; ++b) {
+                    const uint4 eb = entries(b, sub + 8);
+                    group(ea, b, sub, add0);
+                    ea = entries(b + 1, sub);
+                    group(eb, b, sub + 8, [&](R px, R py, R pz) { f1x.add(px); f1y.add(py); f1z.add(pz); });
+                }
+            } else {
+                for (int b = 0; b < bmax; ++b) {
+                    const uint4 eb = entries(b + 1, sub);
+                    group(ea, b, sub, add0);
+                    ea = eb;
+                }
+            }
+        } else if constexpr (LPA == 32) {
+            const int v = lane & 15, half = lane >> 4;
+            uint4 ea = entries(half, v);
+            for (int b = 0; b < nblk; b += 2) {
+                const uint4 en4 = entries(b + 2 + half, v);
+                group(ea, b + half, v, [&](R px, R py, R pz) {
+                    const R qx = __shfl_down_sync(0xffffffffu, px, 16), qy = __shfl_down_sync(0xffffffffu, py, 16),
+                            qz = __shfl_down_sync(0xffffffffu, pz, 16);
+                    add0(px, py, pz);
+                    add0(qx, qy, qz);
+                });
+                ea = en4;
+            }
+        } else {
+            constexpr int NB = LPA / kCols;  // blocks of a round
+            __shared__ R gs[NB][3][kCols];
+            const int v = sub & 15, gb = sub >> 4;
+            uint4 ea = entries(gb, v);
+            for (int b = 0; b < nblk; b += NB) {
+                const uint4 en4 = entries(b + NB + gb, v);
+                R sx3[3] = {0, 0, 0};
+                group(ea, b + gb, v, [&](R px, R py, R pz) { sx3[0] = px; sx3[1] = py; sx3[2] = pz; });
+#pragma unroll
+                for (int c = 0; c < 3; ++c) gs[gb][c][v] = sx3[c];
+                __syncthreads();
+                if (threadIdx.x < 48)
+                    for (int t = 0; t < min(NB, nblk - b); ++t) fx.add(gs[t][threadIdx.x >> 4][v]);
+                __syncthreads();
+                ea = en4;
+            }
         }
     }
-    fx.template group_reduce<LPA>(); fy.template group_reduce<LPA>(); fz.template group_reduce<LPA>();
+    // the bead-atom's force: component c is left complete on its lane (see reduce3)
+    int c = comp_of_lane<LW>(lane & (LW - 1));
+    ACC fsum;
+    if constexpr (LPA == 128) {
+        // (the columns' sums are already split by component: thread 16 comp + column)
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) exchange_add(fx, fx, o);
+        __shared__ ACC total[3];
+        if (n == 0) __syncthreads();  // (no round has passed since the last unit read it; one bead-atom: uniform)
+        if (threadIdx.x < 48 && (threadIdx.x & 15) == 0) total[threadIdx.x >> 4] = fx;
+        __syncthreads();
+        fsum = total[min(c, 2)];
+    } else {
+        if constexpr (LPA == 8) {
+            add_acc(fx, f1x); add_acc(fy, f1y); add_acc(fz, f1z);
+        }
+        fsum = reduce3<LW>(fx, fy, fz, lane & (LW - 1));
+    }
+    if (LPA > 16 && (threadIdx.x & (LPA - 1)) >= 16) c = 3;  // the first 16 lanes keep the books
     // recorded steps: the FP64 form sums its partials in FP64; the FP32 form in
     // float-float on the FP32 pipe (this GPU's FP64 rate is a small fraction of
     // its FP32 rate), kc and mc being a component lane's kinetic energy and momentum
@@ -1049,10 +1235,10 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
     for (int q = 0; q < kNQ; ++q) acc[q] = 0.0;
     float kc = 0.f, kl = 0.f, mc = 0.f, ml = 0.f;  // float-float (hi, lo)
     if (REC && rec) {
-        en = group_sum<LPA>(en);
-        w0 = group_sum<LPA>(w0); w1 = group_sum<LPA>(w1); w2 = group_sum<LPA>(w2);
-        w3 = group_sum<LPA>(w3); w4 = group_sum<LPA>(w4); w5 = group_sum<LPA>(w5);
-        if (!kFF && act && sub == 0) {
+        en = group_sum<LW>(en);
+        w0 = group_sum<LW>(w0); w1 = group_sum<LW>(w1); w2 = group_sum<LW>(w2);
+        w3 = group_sum<LW>(w3); w4 = group_sum<LW>(w4); w5 = group_sum<LW>(w5);
+        if (!kFF && act && (lane & (LW - 1)) == 0) {
             acc[Q_V] = 0.5 * (double)en;
             acc[Q_VIR + 0] = 0.5 * (double)w0; acc[Q_VIR + 1] = 0.5 * (double)w1;
             acc[Q_VIR + 2] = 0.5 * (double)w2; acc[Q_VIR + 3] = 0.5 * (double)w3;
@@ -1060,10 +1246,9 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
         }
     }
     R dd = 0;  // squared displacement component since the last rebuild (ADV)
-    if (act && sub < 3) {
-        const int c = sub;
+    if (act && c < 3) {
         const R invP = sizeof(R) == 4 ? (R)S.invP_f : (R)S.invP;
-        const R fc = (R)(c == 0 ? fx.value() : c == 1 ? fy.value() : fz.value()) * invP;
+        const R fc = (R)fsum.value() * invP;
         R *Fo = reinterpret_cast<R *>(d.f);
         R *V = reinterpret_cast<R *>(d.v);
         const size_t o = (size_t)c * G + gi;
@@ -1109,16 +1294,16 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
             const float fsc = S.fix_scale[c];
             const PS xn = PosT<PM, R>::add(X[o], qq, S.box[c], fsc, S.fix_inv[c]);
             X[o] = xn;
-            reinterpret_cast<PS *>(d.pos[cur ^ 1])[4 * (size_t)gi + c] = xn;
+            reinterpret_cast<PS *>(d.pos[cur ^ 1])[4 * ((size_t)RP.g0 + sl) + c] = pack_pos(xn, MI ? 2 : 0);
             const R dc = PosT<PM, R>::diff(xn, reinterpret_cast<const PS *>(d.xref)[o], fsc);
             dd = dc * dc;
         }
         if (kick || ADV) V[o] = v;
     }
     if (ADV) {
-        const int b0 = grp * LPA;
-        const R tot = __shfl_sync(0xffffffffu, dd, b0) + __shfl_sync(0xffffffffu, dd, b0 + 1) +
-                      __shfl_sync(0xffffffffu, dd, b0 + 2);
+        const int b0 = lane & ~(LW - 1);
+        const R tot = __shfl_sync(0xffffffffu, dd, b0) + __shfl_sync(0xffffffffu, dd, b0 + LW / 4) +
+                      __shfl_sync(0xffffffffu, dd, b0 + LW / 2);
         const R lim = sizeof(R) == 4 ? (R)S.skin2_f : (R)S.skin2;
         if (__any_sync(0xffffffffu, act && sub == 0 && tot > lim) && lane == 0) {
             atomicOr(&d.rflag[(cur ^ 1) * d.nsys + RP.sys], 1u);
@@ -1127,7 +1312,7 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
     }
     if (REC && rec) {
         if constexpr (kFF) {
-            cta_store_partials_ff<LPA>(act && sub == 0, en, w0, w1, w2, w3, w4, w5, kc, kl, mc, ml, red,
+            cta_store_partials_ff<LW>(act && (lane & (LW - 1)) == 0, en, w0, w1, w2, w3, w4, w5, kc, kl, mc, ml, red,
                                        reinterpret_cast<float2 *>(d.part) + (size_t)u * kNQ);
         } else {
 #pragma unroll
@@ -1202,20 +1387,21 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
 // of k_integrate's, operation for operation, so that a fused step gives the
 // same bits as an integrator launch would.  j1 is the next step (its noise row),
 // nxt its position buffer.
-template <int PM, class R, int LPA>
+template <int PM, class R>
 __device__ void npt_next_half(const Dev &d, int j1, int nxt)
 {
     typedef typename PosT<PM, R>::S PS;
-    constexpr int NA = list_atoms(LPA);
+    constexpr int NA = list_atoms(16);
     __shared__ R sdd[3 * NA];
     const size_t G = (size_t)d.G;
-    for (int u = blockIdx.x; u < d.nunits; u += gridDim.x) {
-        const DRep RP = d.rep[d.lcta_rep[u]];
+    for (int u = blockIdx.x; u < d.nunits_rec; u += gridDim.x) {
+        const int2 unit = d.units_rec[u];
+        const DRep RP = d.rep[unit.x];
         const int s = RP.sys;
         const DSys &S = d.sys[s];
         const DNpt *NC = d.npt + s;
         const int t = threadIdx.x, k = t / 3, c = t - 3 * k;
-        const int i = (u - RP.fcta0) * NA + k;
+        const int i = unit.y + k;
         const bool act = t < 3 * NA && i < RP.N;
         R dd = 0;
         if (act) {
@@ -1238,7 +1424,7 @@ __device__ void npt_next_half(const Dev &d, int j1, int nxt)
             const float fsc = S.fix_scale[c];
             const PS xn = PosT<PM, R>::add(X[o], disp, S.box[c], fsc, S.fix_inv[c]);
             X[o] = xn;
-            reinterpret_cast<PS *>(d.pos[nxt])[4 * gi + c] = xn;
+            reinterpret_cast<PS *>(d.pos[nxt])[4 * ((size_t)RP.g0 + d.slot[gi]) + c] = xn;  // (never the shifted form)
             const R dc = PosT<PM, R>::diff(xn, reinterpret_cast<const PS *>(d.xref)[o], fsc);
             dd = dc * dc;
         }
@@ -1264,21 +1450,25 @@ __device__ void npt_next_half(const Dev &d, int j1, int nxt)
 // When the producer of this step's positions requested a rebuild (flag[cur]),
 // the grid first bins, sorts and builds the lists, phases separated by grid
 // barriers.  Dynamic shared memory: the staging chunk of the list build
-// (stage_cap entries; also the sort keys).  FP32 form: at least 7 CTAs per SM
-// (72 registers, no spills; 1064 resident CTAs hold the 1000 units of an
-// 8000-ion crystal in one wave): 5 % faster there than 8 CTAs at 64 registers,
-// no slower on larger systems; six or eight entries in flight per lane spill.
+// (stage_cap entries; also the sort keys).  FP32 form: at least 7 CTAs per SM (72
+// registers; 1064 resident CTAs hold the 1000 units of an 8000-ion crystal in one
+// wave; at 8 the fused variant spills and takes 24 % longer there, the plain one
+// gains 1.6 % on 2 million bead-atoms and loses 7 % on 13824); 6 for 8 lanes in the
+// fused variant, whose second column's sums would spill (13824 ions: 14.9 us instead
+// of 17.9).  Fetching the next group's positions ahead costs more in registers than it
+// hides (6-12 % slower at 6 or 7 CTAs); two groups per loop iteration spill (8000 ions
+// 11.3 us instead of 10.7).
 // The recording variants (energy and virial as well) take 4 CTAs per SM and
 // spill nothing: 10 % faster per step on an isothermal-isobaric run, which
 // records every step, and no slower on the 8000-ion crystal's recorded step.
-template <int PM, class R, int ADV, int REC, int LPA, int MI>
-__global__ void __launch_bounds__(32 * kListWarps, sizeof(R) == 4 ? (REC ? 4 : 7) : 4)
+template <int PM, class R, int ADV, int REC, int LPA, int VAR>
+__global__ void __launch_bounds__(32 * kListWarps, sizeof(R) == 4 ? (REC ? 4 : LPA == 8 && ADV ? 6 : 7) : 4)
     k_step(Dev d, PairTabT<R> T, int kick, int j, int cur)
 {
     extern __shared__ __align__(32) unsigned char fsm[];
     __shared__ BuildSmem B;
     __shared__ PairRow<R> ptab[kMaxTypes * kMaxTypes];
-    if (threadIdx.x < kMaxTypes * kMaxTypes) ptab[threadIdx.x] = pair_row(T, threadIdx.x);
+    if (threadIdx.x < kMaxTypes * kMaxTypes) ptab[threadIdx.x] = pair_row<VAR>(T, threadIdx.x);
     __syncthreads();
     __shared__ double red[kListWarps][kNQ];
     __shared__ double rsh[kListWarps][kNQ + 1];
@@ -1293,13 +1483,14 @@ __global__ void __launch_bounds__(32 * kListWarps, sizeof(R) == 4 ? (REC ? 4 : 7
             d.flag[cur] = 0u;  // this step's rebuild request is consumed
             atomicAdd(d.nrebuild, 1ull);
         }
+        scan_phase(d, cur, B.soff);
         sort_phase<PM>(d, cur, reinterpret_cast<int *>(fsm));
         grid_barrier(d);
         for (int s = 0; s < d.nsys; ++s) {  // the cells of the requesting systems
             if (!d.rebuild_all && d.rflag[cur * d.nsys + s] == 0u) continue;  // uniform over the grid
             const int c0 = d.sys[s].cell0, c1 = d.sys[s].cell1, nb = (int)gridDim.x;
             for (int cell = c0 + (((int)blockIdx.x - c0) % nb + nb) % nb; cell < c1; cell += nb)
-                build_cell<PM, R>(d, T.rc2, sizeof(R) == 4 ? (R)d.sys[s].rl2_f : (R)d.sys[s].rl2, cell, fsm, B);
+                build_cell<PM, R>(d, T.rc2, sizeof(R) == 4 ? (R)d.sys[s].rl2_f : (R)d.sys[s].rl2, cell, cur, fsm, B);
         }
         grid_barrier(d);
         // the per-system requests were read by every phase: consumed now (their
@@ -1313,26 +1504,42 @@ __global__ void __launch_bounds__(32 * kListWarps, sizeof(R) == 4 ? (REC ? 4 : 7
             }
     }
     release_next_step();
-    for (int u = blockIdx.x; u < d.nunits; u += gridDim.x)
-        force_unit<PM, R, ADV, REC, LPA, MI>(d, T, ptab, kick, j, cur, u, red, rsh, s_last);
+    for (int u = blockIdx.x; u < (REC ? d.nunits_rec : d.nunits); u += gridDim.x)
+        force_unit<PM, R, ADV, REC, LPA, VAR>(d, T, ptab, kick, j, cur, u, red, rsh, s_last);
     if constexpr (ADV && REC) {
         // isothermal-isobaric cells: the next step's first half waits for the
         // cells' updates (made by each system's last CTA) behind a grid barrier
         if (d.npt && kick) {
             grid_barrier(d);
-            npt_next_half<PM, R, LPA>(d, j + 1, cur ^ 1);
+            npt_next_half<PM, R>(d, j + 1, cur ^ 1);
         }
     }
 }
 
-template <int PM, class R, int ADV, int REC, int LPA, int MI>
+template <int PM, class R, int ADV, int REC, int LPA, int VAR>
 static cudaError_t step_prepare_one(size_t smem, int nsm, int &grid)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_step<PM, R, ADV, REC, LPA, MI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_step<PM, R, ADV, REC, LPA, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<PM, R, ADV, REC, LPA, MI>, 32 * kListWarps, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<PM, R, ADV, REC, LPA, VAR>, 32 * kListWarps, smem);
     grid = per_sm * nsm;
+    return e;
+}
+
+// attributes and resident grid of the variants one lane count has (see step_any)
+template <int PM, class R, int LPA, int VAR>
+static cudaError_t step_prepare_variant(MdLaunch &m, int nsm)
+{
+    cudaError_t e = cudaSuccess;
+    if (LPA == m.lanes) {
+        e = step_prepare_one<PM, R, 0, 0, LPA, VAR>(m.step_smem, nsm, m.step_grid[0]);
+        if (e == cudaSuccess) e = step_prepare_one<PM, R, 1, 0, LPA, VAR>(m.step_smem, nsm, m.step_grid[2]);
+    }
+    if constexpr (LPA == 16) {
+        if (e == cudaSuccess) e = step_prepare_one<PM, R, 0, 1, 16, VAR>(m.step_smem, nsm, m.step_grid[1]);
+        if (e == cudaSuccess) e = step_prepare_one<PM, R, 1, 1, 16, VAR>(m.step_smem, nsm, m.step_grid[3]);
+    }
     return e;
 }
 
@@ -1344,31 +1551,18 @@ static cudaError_t step_prepare_lanes(MdLaunch &m, int stage_entries)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     m.step_smem = (size_t)stage_entries * (m.mixed ? sizeof(int4) : sizeof(D4));
-    if (m.mixed && m.minimg) {
-        if ((e = step_prepare_one<PM_FIX, float, 0, 0, LPA, 1>(m.step_smem, nsm, m.step_grid[0])) != cudaSuccess) return e;
-        if ((e = step_prepare_one<PM_FIX, float, 0, 1, LPA, 1>(m.step_smem, nsm, m.step_grid[1])) != cudaSuccess) return e;
-        if ((e = step_prepare_one<PM_FIX, float, 1, 0, LPA, 1>(m.step_smem, nsm, m.step_grid[2])) != cudaSuccess) return e;
-        e = step_prepare_one<PM_FIX, float, 1, 1, LPA, 1>(m.step_smem, nsm, m.step_grid[3]);
-    } else if (m.mixed) {
-        if ((e = step_prepare_one<PM_FIX, float, 0, 0, LPA, 0>(m.step_smem, nsm, m.step_grid[0])) != cudaSuccess) return e;
-        if ((e = step_prepare_one<PM_FIX, float, 0, 1, LPA, 0>(m.step_smem, nsm, m.step_grid[1])) != cudaSuccess) return e;
-        if ((e = step_prepare_one<PM_FIX, float, 1, 0, LPA, 0>(m.step_smem, nsm, m.step_grid[2])) != cudaSuccess) return e;
-        e = step_prepare_one<PM_FIX, float, 1, 1, LPA, 0>(m.step_smem, nsm, m.step_grid[3]);
-    } else {
-        if ((e = step_prepare_one<PM_BOX64, double, 0, 0, LPA, 0>(m.step_smem, nsm, m.step_grid[0])) != cudaSuccess) return e;
-        if ((e = step_prepare_one<PM_BOX64, double, 0, 1, LPA, 0>(m.step_smem, nsm, m.step_grid[1])) != cudaSuccess) return e;
-        if ((e = step_prepare_one<PM_BOX64, double, 1, 0, LPA, 0>(m.step_smem, nsm, m.step_grid[2])) != cudaSuccess) return e;
-        e = step_prepare_one<PM_BOX64, double, 1, 1, LPA, 0>(m.step_smem, nsm, m.step_grid[3]);
-    }
-    return e;
+    if (!m.mixed) return step_prepare_variant<PM_BOX64, double, LPA, 0>(m, nsm);
+    if (m.variant == 2) return step_prepare_variant<PM_FIX, float, LPA, 2>(m, nsm);
+    if (m.variant == 1) return step_prepare_variant<PM_FIX, float, LPA, 1>(m, nsm);
+    return step_prepare_variant<PM_FIX, float, LPA, 0>(m, nsm);
 }
 
 // cooperative launch: all CTAs resident at once (the grid barriers need it)
-template <int PM, class R, int ADV, int REC, int LPA, int MI>
+template <int PM, class R, int ADV, int REC, int LPA, int VAR>
 static cudaError_t step_launch(const Dev &d, const MdLaunch &m, const PairTabT<R> &T, int kick, int j, int cur,
                                cudaStream_t st)
 {
-    const int grid = std::min(d.nunits, m.step_grid[ADV * 2 + REC]);
+    const int grid = std::min(REC ? d.nunits_rec : d.nunits, m.step_grid[ADV * 2 + REC]);
     if (grid < 1) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -1382,17 +1576,22 @@ static cudaError_t step_launch(const Dev &d, const MdLaunch &m, const PairTabT<R
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_step<PM, R, ADV, REC, LPA, MI>, d, T, kick, j, cur);
+    return cudaLaunchKernelEx(&cfg, k_step<PM, R, ADV, REC, LPA, VAR>, d, T, kick, j, cur);
 }
 
-template <int PM, class R, int LPA, int MI>
+// steps that may be recorded always run with 16 lanes, whose sums of energies and
+// virials the records are made of, whatever lane count the others have
+template <int PM, class R, int LPA, int VAR>
 static cudaError_t step_any(const Dev &d, const MdLaunch &m, const PairTabT<R> &T, int kick, int j, int cur, int adv,
                             int rec, cudaStream_t st)
 {
-    if (adv && rec) return step_launch<PM, R, 1, 1, LPA, MI>(d, m, T, kick, j, cur, st);
-    if (adv) return step_launch<PM, R, 1, 0, LPA, MI>(d, m, T, kick, j, cur, st);
-    if (rec) return step_launch<PM, R, 0, 1, LPA, MI>(d, m, T, kick, j, cur, st);
-    return step_launch<PM, R, 0, 0, LPA, MI>(d, m, T, kick, j, cur, st);
+    if constexpr (LPA == 16) {
+        if (adv && rec) return step_launch<PM, R, 1, 1, 16, VAR>(d, m, T, kick, j, cur, st);
+        if (rec) return step_launch<PM, R, 0, 1, 16, VAR>(d, m, T, kick, j, cur, st);
+    }
+    if (rec) return cudaErrorInvalidValue;
+    if (adv) return step_launch<PM, R, 1, 0, LPA, VAR>(d, m, T, kick, j, cur, st);
+    return step_launch<PM, R, 0, 0, LPA, VAR>(d, m, T, kick, j, cur, st);
 }
 
 // the step kernel of one lane count (one translation unit per count)
@@ -1401,7 +1600,8 @@ static cudaError_t step_force_lanes(const Dev &d, const MdLaunch &m, const PairT
                                     const PairTabT<double> &Td, int kick, int j, int cur, int adv, int rec,
                                     cudaStream_t st)
 {
-    if (m.mixed && m.minimg) return step_any<PM_FIX, float, LPA, 1>(d, m, Tf, kick, j, cur, adv, rec, st);
+    if (m.mixed && m.variant == 2) return step_any<PM_FIX, float, LPA, 2>(d, m, Tf, kick, j, cur, adv, rec, st);
+    if (m.mixed && m.variant == 1) return step_any<PM_FIX, float, LPA, 1>(d, m, Tf, kick, j, cur, adv, rec, st);
     if (m.mixed) return step_any<PM_FIX, float, LPA, 0>(d, m, Tf, kick, j, cur, adv, rec, st);
     return step_any<PM_BOX64, double, LPA, 0>(d, m, Td, kick, j, cur, adv, rec, st);
 }

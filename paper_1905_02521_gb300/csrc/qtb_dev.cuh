@@ -24,6 +24,7 @@ constexpr int kNQ = 16;              // partial sums per CTA (see Q_* below)
 constexpr int kRedGroup = 16;        // force units per group of the two-level record reduction
 constexpr int kFixBits = 30;         // fixed-point positions: box edge = 2^30 units
 constexpr int kMaxTypes = 4;
+constexpr int kFitN = 10;            // coefficients of the FP32 Coulomb fits (degree 9)
 constexpr int kWarpsPerForceCta = 8;  // warps of the list build kernel
 
 // partial-sum slots
@@ -67,14 +68,20 @@ struct DNpt {
     float lam_oldf, inv_lamf;
 };
 
-// Neighbour-list entry (32 bits): replica-local index j in bits 0..25, the
-// periodic image m of the entry (per component m mod 4, two bits each: x at
-// bit 26, y at 28, z at 30).  With 30-bit fixed point the image shift is
-// (m mod 4) * 2^30, exact in wrapping 32-bit arithmetic.
+// Neighbour-list entry (32 bits): replica-local slot of bead-atom j in the packed
+// positions in bits 0..25, the periodic image m of the entry (per component m mod
+// 4, two bits each: x at bit 26, y at 28, z at 30).  With 30-bit fixed point the
+// image shift is (m mod 4) * 2^30, exact in wrapping 32-bit arithmetic.  The
+// minimum-image variant of the step kernel needs no image: its entries are the
+// byte offset of j's packed position, 16 slot.
 constexpr unsigned kNbIdx = (1u << 26) - 1u;
+// A list is stored in blocks of 16 columns of 4 entries: entry k = 64 b + 16 q + v
+// (block b, column v < 16, q < 4) at 64 b + 4 v + q, so that one 16-byte load brings a
+// lane of the step kernel a column.
+constexpr int kCols = 16, kColNE = 4, kColBlock = kCols * kColNE;
 constexpr int kMaxCellCap = 512;        // slots per cell of the cell list
 constexpr int kListWarps = 4;        // warps per CTA of the list force kernel
-// lanes per home bead-atom of the step kernel: 8, 16 (default) or 32; a force
+// lanes per home bead-atom of the step kernel: 8, 16, 32 or 128; a force
 // unit (one CTA's share of work) holds list_atoms(lanes) bead-atoms
 __host__ __device__ constexpr int list_atoms(int lanes) { return kListWarps * 32 / lanes; }
 
@@ -87,7 +94,7 @@ struct DSys {
     int taps0;         // offset of h_0 in the taps arrays
     int rep0;          // first replica (pair potential)
     int icta0, icta1;  // integrator CTA range
-    int fcta0, fcta1;  // force CTA range
+    int fcta0, fcta1;  // force CTA range (pair potential: of the 16-lane units)
     int grp0, ngrp;    // its groups of kRedGroup force units (two-level record reduction)
     int ccta0, ccta1;  // centroid-estimator CTA range (empty for one bead)
     int cell0, cell1;  // cells of all its replicas (pair potential)
@@ -138,6 +145,11 @@ template <class R> struct PairTabT {
     R alpha2_l2e, erfc_us;
     R rl2;                            // (r_cut + skin)^2: neighbour-list radius
     R erfc_c[12];
+    // FP32 form, variants 1 and 2 of the step kernel: with x = alpha r and u = r^2 r2_us - 1,
+    // the Chebyshev fits (monomials in u) of -alpha^3 (erf x - 2 x e^{-x^2}/sqrt(pi))/x^3 (cf)
+    // and alpha erf(x)/x (ce); nl2e_rho = -log2(e)/rho
+    R r2_us, cf[kFitN], ce[kFitN];
+    R nl2e_rho[kMaxTypes * kMaxTypes];
     R hdt_m[kMaxTypes];               // dt / (2 m mvv2e)
     R ext_k[kMaxTypes];               // HARMONIC: m mvv2e w0^2
     R ext_V0, ext_ia2;                // DOUBLEWELL: V0, 1/a^2
@@ -161,8 +173,10 @@ struct Dev {
     const DSys *sys;
     const DRep *rep;
     const int *cell_rep;  // [ncells]
-    const int *lcta_rep;  // [nunits] replica of each force unit
-    int nunits;           // force units
+    // force units, a CTA's share of the bead-atoms: (replica, first atom).  units: of the
+    // context's lane count; units_rec: of the 16-lane variants that may record a step
+    const int2 *units, *units_rec;
+    int nunits, nunits_rec;
     const int *icta_sys;  // [integrator CTAs] system of each CTA
     const int *ext_cta_sys;
     // state
@@ -176,9 +190,17 @@ struct Dev {
     int *cidx;            // [ncells * cap] bead-atom index, sorted
     void *cpos;           // [ncells * cap] packed {x, y, z, replica-local index} (int4 or 4 doubles)
     // neighbour lists (pair potential)
-    void *pos[2];         // [G] packed {x, y, z, type} (int4 or 4 doubles); step s reads pos[s & 1]
+    // packed positions {x, y, z, type} (int4 or 4 doubles), [G] in slot order (replica
+    // by replica, in the order of the cells of the last rebuild, so that the gathers of
+    // a list run over whole cache lines); step s reads pos[s & 1].  Fixed-point
+    // coordinates are stored shifted left by pshift (2 in the minimum-image variant:
+    // full 32-bit fractions of the edge, whose differences wrap to the minimum image).
+    void *pos[2];
+    int *slot;            // [G] replica-local slot of each bead-atom
+    int *cbase;           // [ncells] first slot of each cell
+    int pshift;
     void *xref;           // [3][G] positions at the last rebuild (type of x)
-    unsigned *nbr;        // [G][maxnb] list entries (see kNbIdx)
+    unsigned *nbr;        // [G][maxnb] list entries (see kNbIdx, kCols)
     int *nnb;             // [G] entries per bead-atom
     int maxnb;
     unsigned *flag;       // [2] rebuild requests; flag[s & 1] is set by whoever produces the positions of step s

@@ -58,10 +58,12 @@ struct MdLaunch {
     int fused;            // all systems one-bead with a pair potential: the step kernel
                           // carries out the first half of the next step
     int nm_big;           // ring-polymer integrator with 32 atoms per CTA (large contexts)
-    int lanes;            // lanes per bead-atom of the step kernel (8, 16, 32)
+    int lanes;            // lanes per bead-atom of the step kernel of steps that are not recorded (8, 16, 32, 128)
     int step_grid[4];     // resident CTAs of the step kernel, by (adv, rec)
-    int minimg;           // mixed form, fixed cells all larger than 2 (r_cut + 2 skin): the step
-                          // kernel variant that takes list displacements by minimum image
+    int variant;          // step kernel variant of the mixed form: 0 any alpha r_cut (exponential and
+                          // erfc polynomial), 1 the Coulomb term as one polynomial in r^2, 2 the
+                          // same with list displacements by minimum image (fixed cells all larger
+                          // than 2 (r_cut + 2 skin))
     size_t step_smem;     // its dynamic shared memory (list build staging chunk)
 };
 constexpr int kIntAtomsPerWarp = 10;                   // integrator: lanes 3a + c, a < 10
@@ -69,15 +71,18 @@ constexpr int kIntAtomsPerCta = 4 * kIntAtomsPerWarp;  // 128 threads
 constexpr int kStencilCells = 125;                     // 5^3 stencil of (r_cut + skin)/2 cells
 // attributes and resident grid sizes of the cooperative step kernel (m.lanes)
 cudaError_t step_prepare(MdLaunch &m, int stage_entries);
-// per lane count, one translation unit each (md_step8.cu, md_step16.cu, md_step32.cu)
+// per lane count, one translation unit each (md_step8.cu .. md_step128.cu)
 cudaError_t step_prepare_l8(MdLaunch &m, int stage_entries);
 cudaError_t step_prepare_l16(MdLaunch &m, int stage_entries);
 cudaError_t step_prepare_l32(MdLaunch &m, int stage_entries);
+cudaError_t step_prepare_l128(MdLaunch &m, int stage_entries);
 cudaError_t step_force_l8(const Dev &d, const MdLaunch &m, const PairTabT<float> &Tf, const PairTabT<double> &Td,
                           int kick, int j, int cur, int adv, int rec, cudaStream_t st);
 cudaError_t step_force_l16(const Dev &d, const MdLaunch &m, const PairTabT<float> &Tf, const PairTabT<double> &Td,
                            int kick, int j, int cur, int adv, int rec, cudaStream_t st);
 cudaError_t step_force_l32(const Dev &d, const MdLaunch &m, const PairTabT<float> &Tf, const PairTabT<double> &Td,
+                           int kick, int j, int cur, int adv, int rec, cudaStream_t st);
+cudaError_t step_force_l128(const Dev &d, const MdLaunch &m, const PairTabT<float> &Tf, const PairTabT<double> &Td,
                            int kick, int j, int cur, int adv, int rec, cudaStream_t st);
 // positions of step s: the integrator writes pos[cur], cur = s & 1, and
 // requests a list rebuild in flag[cur] when some bead-atom moved skin/2

@@ -8,6 +8,7 @@
 #include <cuda.h>
 #include <dlfcn.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -63,6 +64,7 @@ struct qtb_ctx {
     std::vector<double> skins;   // each system's skin, A
     qtb_params p{};
     std::vector<double> mass, charge, bA, brho, bC;
+    std::vector<char> ring_kind;  // per system: the ring holds spectra
     bool mixed = false, pair = true;
     int fk = FK_FP64;  // ring / filter arithmetic
     size_t rsz = 8;    // sizeof(R)
@@ -92,6 +94,10 @@ struct qtb_ctx {
     int Kmax = 0;
     int max_dofp = 0, max_repN = 0;
     size_t ring_bytes = 0;
+    bool fft = false;              // some system's FP64 filter is a fast convolution
+    bool direct = true;            // some system's is not
+    void *d_fft = nullptr;         // its tables
+    size_t fft_bytes = 0;
     std::vector<void *> allocs;
     std::map<int, double *> kappaF;  // P -> device F grid
     double *dS = nullptr;            // spectrum scratch
@@ -375,14 +381,17 @@ int refresh_forces(qtb_ctx *c)
 
 void gen_white(qtb_ctx *c, long long blk)
 {
-    launch_white(c->d, c->fk, c->max_dofp, c->d.nsys, blk, c->st);
+    if (c->fft) launch_white_fft(c->d, c->max_dofp, blk, c->st);
+    if (c->direct) launch_white(c->d, c->fk, c->max_dofp, c->d.nsys, blk, c->st);
 }
 
 void filter_block(qtb_ctx *c)
 {
     if (c->fk == FK_BF16)
         launch_filter_tc(c->d, &c->tmA, &c->tmB, c->n_tiles, c->d_tiles, c->st);
-    else
+    else if (c->fft)
+        launch_filter_fft(c->d, c->max_dofp, c->st);
+    if (c->fk != FK_BF16 && c->direct)
         launch_filter_simt(c->d, c->fk, c->max_dofp, c->d.nsys, c->Kmax, c->st);
 }
 
@@ -666,6 +675,11 @@ int setup_fourier(qtb_ctx *c, const std::vector<DSpec> &spec)
     return QTB_OK;
 }
 
+// The FP64 filter of a system switches to the fast convolution at this half
+// length, as long as its spectra stay within the limit.
+constexpr int kFftMinK = 64;
+constexpr size_t kFftMaxRing = (size_t)16 << 30;
+
 // (re)build taps of every system from hs[].mode/n_taps/omega_max
 int rebuild_filters(qtb_ctx *c)
 {
@@ -724,16 +738,46 @@ int rebuild_filters(qtb_ctx *c)
     const int Kb = (Kmax + kBlockSteps - 1) / kBlockSteps;
     const int nslots = 2 * Kb + 1;
     const size_t esz = (c->fk == FK_FP64) ? 8 : (c->fk == FK_FP32 ? 4 : 2);
-    const size_t need = esz * (size_t)nslots * (size_t)c->d.Dtot * kBlockSteps;
-    if (need > c->ring_bytes || nslots != c->d.nslots) {
-        if (need > c->ring_bytes) {
-            c->release(c->d.ring);
-            c->d.ring = c->alloc(need);
-            if (!c->d.ring) return fail(QTB_ERR_OOM, "noise ring allocation (%zu bytes) failed", need);
-            c->ring_bytes = need;
+    // systems with taps long enough for the fast convolution; its spectra take twice
+    // the ring (a context whose device memory does not hold that filters directly)
+    const size_t need256 = esz * (size_t)nslots * (size_t)c->d.Dtot * kBlockSteps;
+    bool fft = false;
+    for (int s = 0; s < ns; ++s) {
+        c->ds[s].fft = c->fk == FK_FP64 && c->gen == QTB_GEN_FILTER && c->ds[s].K >= kFftMinK &&
+                       2 * esz * (size_t)(2 * ((c->ds[s].K + kBlockSteps - 1) / kBlockSteps) + 1) * (size_t)c->ds[s].dofp * kBlockSteps <= kFftMaxRing;
+        fft = fft || c->ds[s].fft;
+    }
+    int row = fft ? 2 * kBlockSteps : kBlockSteps;
+    if (fft && 2 * need256 > c->ring_bytes) {
+        c->release(c->d.ring);
+        c->ring_bytes = 0;
+        c->d.ring = c->alloc(2 * need256);
+        if (c->d.ring) {
+            c->ring_bytes = 2 * need256;
+        } else {
+            cudaGetLastError();
+            for (int s = 0; s < ns; ++s) c->ds[s].fft = 0;
+            fft = false;
+            row = kBlockSteps;
         }
         c->ring_hi = c->ring_lo = LLONG_MIN;
     }
+    if (need256 > c->ring_bytes) {
+        c->release(c->d.ring);
+        c->ring_bytes = 0;
+        c->d.ring = c->alloc(need256);
+        if (!c->d.ring) return fail(QTB_ERR_OOM, "noise ring allocation (%zu bytes) failed", need256);
+        c->ring_bytes = need256;
+        c->ring_hi = c->ring_lo = LLONG_MIN;
+    }
+    // which systems' rows are spectra decides what the ring's blocks hold
+    std::vector<char> kind(ns);
+    for (int s = 0; s < ns; ++s) kind[s] = (char)c->ds[s].fft;
+    if (nslots != c->d.nslots || row != c->d.ring_row || kind != c->ring_kind) c->ring_hi = c->ring_lo = LLONG_MIN;
+    c->ring_kind = kind;
+    c->d.ring_row = row;
+    c->direct = std::find(kind.begin(), kind.end(), 0) != kind.end();
+    c->fft = fft;
     c->d.Kb = Kb;
     c->d.nslots = nslots;
     c->Kmax = Kmax;
@@ -741,6 +785,20 @@ int rebuild_filters(qtb_ctx *c)
     c->d.taps64 = c->d_taps64;
     c->d.tapsR = (c->fk == FK_FP64) ? (const void *)c->d_taps64 : (const void *)c->d_taps32;
     CUDA_TRY(cudaMemcpyAsync((void *)c->d.sys, c->ds.data(), sizeof(DSys) * ns, cudaMemcpyHostToDevice, c->st));
+    if (c->fft) {
+        const size_t tb = esz * fft_table_values(nslots, ns);
+        if (tb > c->fft_bytes) {
+            c->release(c->d_fft);
+            c->d_fft = c->alloc(tb);
+            if (!c->d_fft) return fail(QTB_ERR_OOM, "filter spectra allocation failed");
+            c->fft_bytes = tb;
+        }
+        c->d.fft_tw = c->d_fft;
+        c->d.fft_g = (char *)c->d_fft + esz * fft_table_values(0, ns);
+        launch_fft_tables(c->d, c->d_taps64, (void *)c->d.fft_tw, (void *)c->d.fft_g, c->st);
+        CUDA_TRY(cudaGetLastError());
+        CUDA_TRY(filter_fft_prepare());
+    }
     if (c->fk == FK_BF16) {
         int rc = setup_tc(c);
         if (rc) return rc;

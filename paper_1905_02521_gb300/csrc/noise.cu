@@ -12,34 +12,12 @@
 
 #include "qtb_dev.cuh"
 #include "qtb_kernels.cuh"
+#include "qtb_normal.cuh"
 
 namespace qtb {
 
 // ---------------------------------------------------------------------------
-// White noise: one Philox call per (dof, 4 steps); Box-Muller pairs
-// (w0,w1) -> steps 4q, 4q+1 (cos, sin), (w2,w3) -> 4q+2, 4q+3.
-
-__device__ __forceinline__ void bm_pair(uint32_t a, uint32_t b, double &z0, double &z1)
-{
-    double u1 = ((double)a + 1.0) * 2.3283064365386963e-10;  // 2^-32, (0, 1]
-    double u2 = (double)b * 2.3283064365386963e-10;          // [0, 1)
-    double r = sqrt(-2.0 * log(u1));
-    double s, c;
-    sincospi(2.0 * u2, &s, &c);
-    z0 = r * c;
-    z1 = r * s;
-}
-
-__device__ __forceinline__ void bm_pair(uint32_t a, uint32_t b, float &z0, float &z1)
-{
-    float u1 = ((float)a + 1.0f) * 2.3283064365386963e-10f;
-    float u2 = (float)b * 2.3283064365386963e-10f;
-    float r = sqrtf(-2.0f * logf(u1));
-    float s, c;
-    sincospif(2.0f * u2, &s, &c);
-    z0 = r * c;
-    z1 = r * s;
-}
+// White noise: one Philox call per (dof, 4 steps).
 
 template <class T> struct RingStore;
 template <> struct RingStore<double> {
@@ -74,25 +52,17 @@ __global__ void k_white(Dev d, long long blk_override)
     const DSys s = d.sys[blockIdx.y];
     long long local = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     int dofl = (int)(local >> 6), qi = (int)(local & 63);
-    if (dofl >= s.dofp) return;
+    if (dofl >= s.dofp || s.fft) return;
     long long blk = (blk_override == LLONG_MIN) ? d.clock[0] + d.Kb : blk_override;
     int slot = (int)(blk - floor_div(blk, d.nslots) * d.nslots);
-    T *dst = reinterpret_cast<T *>(d.ring) + ((size_t)slot * d.Dtot + s.dof0 + dofl) * kBlockSteps + 4 * qi;
-    C z0 = 0, z1 = 0, z2 = 0, z3 = 0;
-    if (dofl < 3 * s.N * s.P) {
-        long long q = blk * (kBlockSteps / 4) + qi;
-        unsigned long long uq = (unsigned long long)q;
-        uint4 ctr = make_uint4((uint32_t)uq, (uint32_t)dofl, 0u, (uint32_t)(uq >> 32));
-        uint32_t sysid = (uint32_t)blockIdx.y;
-        uint4 w = philox4x32_10(ctr, (uint32_t)d.seed, (uint32_t)(d.seed >> 32) ^ sysid);
-        bm_pair(w.x, w.y, z0, z1);
-        bm_pair(w.z, w.w, z2, z3);
-    }
-    RingStore<T>::put(dst, z0, z1, z2, z3);
+    T *dst = reinterpret_cast<T *>(d.ring) + ((size_t)slot * d.Dtot + s.dof0 + dofl) * d.ring_row + 4 * qi;
+    C z[4] = {0, 0, 0, 0};
+    if (dofl < 3 * s.N * s.P) white4(d, blockIdx.y, dofl, blk * (kBlockSteps / 4) + qi, z);
+    RingStore<T>::put(dst, z[0], z[1], z[2], z[3]);
 }
 
 // ---------------------------------------------------------------------------
-// SIMT filter: one CTA (256 threads = 256 output steps) per dof.
+// SIMT filter (short taps; longer ones: noise_fft.cu): one CTA (256 threads = 256 output steps) per dof.
 // grid = (max dofp, nsys); dynamic smem = (256 + 2 Kmax + Kmax + 1) * sizeof(T)
 template <class T>
 __global__ void k_filter_simt(Dev d)
@@ -101,7 +71,7 @@ __global__ void k_filter_simt(Dev d)
     T *win = reinterpret_cast<T *>(smraw);
     const DSys s = d.sys[blockIdx.y];
     int dofl = blockIdx.x;
-    if (dofl >= s.dofp) return;
+    if (dofl >= s.dofp || s.fft) return;
     const int K = s.K, span = kBlockSteps + 2 * K;
     T *h = win + span;
     long long blk = d.clock[0];
@@ -117,7 +87,7 @@ __global__ void k_filter_simt(Dev d)
         long long n = blk * kBlockSteps - K + t;
         long long rb = floor_div(n, kBlockSteps);
         int slot = (int)(rb - floor_div(rb, d.nslots) * d.nslots);
-        win[t] = ring[((size_t)slot * d.Dtot + s.dof0 + dofl) * kBlockSteps + (int)(n - rb * kBlockSteps)];
+        win[t] = ring[((size_t)slot * d.Dtot + s.dof0 + dofl) * d.ring_row + (int)(n - rb * kBlockSteps)];
     }
     for (int t = threadIdx.x; t <= K; t += blockDim.x) h[t] = taps[t];
     __syncthreads();
@@ -125,6 +95,101 @@ __global__ void k_filter_simt(Dev d)
     T acc = h[0] * win[j + K];
     for (int k = 1; k <= K; ++k) acc += h[k] * (win[j + K - k] + win[j + K + k]);
     eta[(size_t)j * d.Dtot + s.dof0 + dofl] = acc;
+}
+
+// FP32 filter of longer taps: the same sums in the same order (bit for bit) with
+// their operands in registers.  A warp takes one dof, a lane 8 consecutive steps; of
+// the window, which slides by one step a tap on either side, four new values a side
+// come with one 16-byte load each four taps, so that 64 of ~75 instructions are the
+// additions and multiply-adds themselves.  The window lies in shared memory with 4
+// words of padding every 32, which puts the lanes' 16-byte loads (32 bytes apart) on
+// different banks.  Measured, 262152 dofs, 2049 taps: 6.4 ms a
+// block instead of 19.5 (k_filter_simt); its instructions alone would take 4.3.
+constexpr int kTileDofs = 8;   // dofs (warps) per CTA: full 32-byte sectors of eta
+constexpr int kTileTaps = 16;  // taps per loop iteration (the register windows rotate in place)
+__host__ __device__ constexpr int tile_taps(int K) { return (K + kTileTaps) / kTileTaps * kTileTaps; }  // 0 .. K, rounded up
+__host__ __device__ constexpr int tile_pad(int i) { return i + 4 * (i >> 5); }
+// words of a window: the steps, 16 of margin a side for the zeros past tap K, alignment
+__host__ __device__ constexpr int tile_window(int K) { return (tile_pad(kBlockSteps + 2 * K + 48) + 7) & ~3; }
+
+__global__ void __launch_bounds__(32 * kTileDofs) k_filter_tile(Dev d, int Kmax)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const DSys s = d.sys[blockIdx.y];
+    const int dof0 = blockIdx.x * kTileDofs;
+    if (dof0 >= s.dofp) return;
+    const int K = s.K, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, dofl = dof0 + warp;
+    float *h = reinterpret_cast<float *>(smraw);         // taps, h_0 and those past K as zeros
+    float *win = h + tile_taps(Kmax) + (size_t)warp * tile_window(Kmax);
+    // step blk 256 + i - K at window index o + i: o + K mod 4 = 3 aligns the loads below
+    const int o = 16 + ((3 - K) & 3), span = kBlockSteps + 2 * K;
+    const float *ring = reinterpret_cast<const float *>(d.ring);
+    const float *taps = reinterpret_cast<const float *>(d.tapsR) + s.taps0;
+    const long long blk = d.clock[0];
+    for (int t = threadIdx.x; t < tile_taps(K); t += blockDim.x) h[t] = t > 0 && t <= K ? taps[t] : 0.0f;
+    for (int q = -d.Kb; q <= d.Kb; ++q) {
+        const long long rb = blk + q;
+        const int slot = (int)(rb - floor_div(rb, d.nslots) * d.nslots);
+        const float *src = ring + ((size_t)slot * d.Dtot + s.dof0 + dofl) * d.ring_row;
+        for (int e = lane; e < kBlockSteps; e += 32) {
+            const int i = q * kBlockSteps + K + e;
+            if (i >= 0 && i < span) win[tile_pad(o + i)] = src[e];
+        }
+    }
+    // the margins that the zeros past tap K meet
+    if (lane < o) win[tile_pad(lane)] = 0.0f;
+    if (lane < 16) win[tile_pad(o + span + lane)] = 0.0f;
+    __syncthreads();
+    const int c = o + 8 * lane + K;  // window index of this lane's first step; c mod 4 = 3
+    // Blocks of four window values: block m of the left side starts at c - 3 - 4 m, of the
+    // right side at c - 3 + 4 m.  Taps 4 m .. 4 m + 3 meet the left blocks m, m - 1, m - 2
+    // and the right ones m .. m + 3; block m lives in slot m mod 4.
+    float acc[8], L[4][4], Rw[4][4];
+    auto load4 = [&](int i, float (&r)[4]) {
+        const float4 v = *reinterpret_cast<const float4 *>(win + tile_pad(i));
+        r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
+    };
+    load4(c - 3 + 4, L[3]);
+    load4(c - 3 + 8, L[2]);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) load4(c - 3 + 4 * m, Rw[m]);
+    const float h0 = taps[0];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = h0 * Rw[(i + 3) >> 2][(i + 3) & 3];
+    for (int k0 = 0; k0 <= K; k0 += kTileTaps) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            load4(c - 3 - k0 - 4 * m, L[m]);
+            load4(c - 3 + k0 + 4 * (m + 3), Rw[(m + 3) & 3]);
+            const float4 hv = *reinterpret_cast<const float4 *>(h + k0 + 4 * m);
+            const float hk[4] = {hv.x, hv.y, hv.z, hv.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int l = i + 3 - k, r = i + 3 + k;
+                    acc[i] = fmaf(hk[k], L[(m - (l >> 2)) & 3][l & 3] + Rw[(m + (r >> 2)) & 3][r & 3], acc[i]);
+                }
+        }
+    }
+    // steps by rows of the CTA's dofs
+    __syncthreads();
+    float *rows = h;  // [256][kTileDofs + 1]
+    const bool real = dofl < 3 * s.N * s.P;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) rows[(8 * lane + i) * (kTileDofs + 1) + warp] = real ? acc[i] : 0.0f;
+    __syncthreads();
+    float *eta = reinterpret_cast<float *>(d.eta) + s.dof0 + dof0;
+    for (int e = threadIdx.x; e < kBlockSteps * kTileDofs; e += blockDim.x) {
+        const int j = e / kTileDofs, l = e % kTileDofs;
+        eta[(size_t)j * d.Dtot + l] = rows[j * (kTileDofs + 1) + l];
+    }
+}
+
+static size_t tile_smem(int Kmax)
+{
+    const size_t w = (size_t)tile_taps(Kmax) + (size_t)kTileDofs * tile_window(Kmax);
+    return 4 * std::max(w, (size_t)kBlockSteps * (kTileDofs + 1));
 }
 
 // ---------------------------------------------------------------------------
@@ -474,16 +539,10 @@ __global__ void __launch_bounds__(256) k_fourier(Dev d, const R *sq, const R *tw
     for (int w = threadIdx.x; w < kSegPairs * 2 * nq; w += blockDim.x) {
         const int q = w % nq, ab = (w / nq) & 1, p = w / (2 * nq);
         const int dofl = dof_first + 2 * p + ab;
-        C z0 = 0, z1 = 0, z2 = 0, z3 = 0;
-        if (dofl < nreal) {
-            const unsigned long long uq = (unsigned long long)(seg * nq + q);
-            uint4 ctr = make_uint4((uint32_t)uq, (uint32_t)dofl, 0u, (uint32_t)(uq >> 32));
-            uint4 r = philox4x32_10(ctr, (uint32_t)d.seed, (uint32_t)(d.seed >> 32) ^ (uint32_t)blockIdx.y);
-            bm_pair(r.x, r.y, z0, z1);
-            bm_pair(r.z, r.w, z2, z3);
-        }
+        C z[4] = {0, 0, 0, 0};
+        if (dofl < nreal) white4(d, blockIdx.y, dofl, seg * nq + q, z);
         R *dst = bufB + p * span + ab * n + 4 * q;
-        dst[0] = (R)z0; dst[1] = (R)z1; dst[2] = (R)z2; dst[3] = (R)z3;
+        dst[0] = (R)z[0]; dst[1] = (R)z[1]; dst[2] = (R)z[2]; dst[3] = (R)z[3];
     }
     __syncthreads();
     // 2) W_j = Z_a,j + i Z_b,j (sq holds sqrt(S_j/n): the 1/sqrt(n) is folded in)
@@ -554,6 +613,11 @@ void launch_white(const Dev &d, int filter_kind, int max_dofp, int nsys, long lo
         k_white<__nv_bfloat16, float><<<grid, 256, 0, st>>>(d, blk);
 }
 
+// the tiled FP32 filter from this half length on (below, the window loads dominate
+// either form), up to what its 8 windows need of shared memory
+constexpr int kTileMinK = 8;
+constexpr size_t kTileMaxSmem = 220 * 1024;
+
 void launch_filter_simt(const Dev &d, int filter_kind, int max_dofp, int nsys, int Kmax, cudaStream_t st)
 {
     dim3 grid((unsigned)max_dofp, (unsigned)nsys);
@@ -562,7 +626,10 @@ void launch_filter_simt(const Dev &d, int filter_kind, int max_dofp, int nsys, i
         k_filter_simt<double><<<grid, kBlockSteps, sm, st>>>(d);
     } else {
         size_t sm = sizeof(float) * (kBlockSteps + 3 * Kmax + 1);
-        k_filter_simt<float><<<grid, kBlockSteps, sm, st>>>(d);
+        if (Kmax >= kTileMinK && tile_smem(Kmax) <= kTileMaxSmem)
+            k_filter_tile<<<dim3((unsigned)(max_dofp / kTileDofs), (unsigned)nsys), 32 * kTileDofs, tile_smem(Kmax), st>>>(d, Kmax);
+        else
+            k_filter_simt<float><<<grid, kBlockSteps, sm, st>>>(d);
     }
 }
 
@@ -571,6 +638,8 @@ cudaError_t filter_simt_prepare(int Kmax)
     size_t sm = sizeof(double) * (kBlockSteps + 3 * Kmax + 1);
     cudaError_t e = cudaFuncSetAttribute(k_filter_simt<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sm);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_filter_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::min(tile_smem(Kmax), kTileMaxSmem));
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_filter_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)(sm / 2 + 16));

@@ -92,6 +92,7 @@ struct DSys {
     int dofp;          // padded dof count of this system (multiple of kDofPad)
     int K;             // filter half length (taps h_0..h_K)
     int taps0;         // offset of h_0 in the taps arrays
+    int fft;           // FP64 filter by fast convolution (noise_fft.cu)
     int rep0;          // first replica (pair potential)
     int icta0, icta1;  // integrator CTA range
     int fcta0, fcta1;  // force CTA range (pair potential: of the 16-lane units)
@@ -210,7 +211,11 @@ struct Dev {
     unsigned long long *nrebuild;  // list rebuilds carried out
     int eta_blocks;       // blocks per noise segment (1: time-domain filter)
     // noise
-    void *ring;           // [nslots][Dtot][256] white noise (double, float or bf16)
+    // white noise [nslots][Dtot][ring_row]: 256 steps of a dof (double, float or bf16) or,
+    // for systems of the fast convolution, 512 complex values per two dofs (ring_row 512)
+    void *ring;
+    int ring_row;
+    const void *fft_g, *fft_tw;  // the filters' spectra [nsys][nslots][512] and twiddles [512] (complex)
     void *eta;            // [256][Dtot] coloured noise (R)
     const double *taps64; // FP64 taps
     const void *tapsR;    // taps in the filter type

@@ -27,6 +27,13 @@ bool kappa_model_accepts(const qtb_kappa_model *M, int P);
 void launch_white(const Dev &d, int filter_kind, int max_dofp, int nsys, long long blk, cudaStream_t st);
 void launch_filter_simt(const Dev &d, int filter_kind, int max_dofp, int nsys, int Kmax, cudaStream_t st);
 cudaError_t filter_simt_prepare(int Kmax);
+// noise_fft.cu: the FP64 filter of long taps by fast convolution (systems with
+// DSys::fft).  Size (in values) of its tables: twiddles, then the filters' spectra
+size_t fft_table_values(int nslots, int nsys);
+cudaError_t filter_fft_prepare();
+void launch_fft_tables(const Dev &d, const double *taps64, void *tw, void *G, cudaStream_t st);
+void launch_white_fft(const Dev &d, int max_dofp, long long blk, cudaStream_t st);
+void launch_filter_fft(const Dev &d, int max_dofp, cudaStream_t st);
 void launch_spectrum_taps(const DSpec *spec, int nsys, int Kmax, double *S, double *h64, float *h32,
                           const float *mlp_w, cudaStream_t st);
 

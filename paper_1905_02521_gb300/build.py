@@ -21,7 +21,7 @@ LIB = os.path.join(LIBDIR, "libqtb.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # the MD sources (md_kernels.cuh, md_integrate.cuh) write every fused multiply-add out explicitly (the integrator and the
 # fused force epilogue must round alike): no automatic contraction there
-EXTRA = {f: ["--fmad=false"] for f in ("md.cu", "md_step8.cu", "md_step16.cu", "md_step32.cu", "md_step128.cu")}
+EXTRA = {f: ["--fmad=false"] for f in ("md.cu", "ext.cu", "md_step8.cu", "md_step16.cu", "md_step32.cu", "md_step128.cu")}
 
 
 def nvcc() -> str:

@@ -73,6 +73,8 @@ struct qtb_ctx {
     std::vector<DRep> dr;
     std::vector<int> cell_rep, icta_sys, ccta_sys;
     std::vector<int2> units, units_rec;  // force units (Dev::units)
+    std::vector<int2> ext_units;         // external-potential units (Dev::ext_units)
+    int ext_rows = 0;                    // records ext_part holds
     Dev d{};
     MdLaunch ml{};
     PairTab tab{};
@@ -493,6 +495,8 @@ void ensure_eta(qtb_ctx *c, long long b)
     c->eta_blk = b;
 }
 
+constexpr long long kExtPartBytes = 64LL << 20;  // record rows of ext.cu per launch
+
 // Profiling: event pairs recorded around each kernel class inside the graph
 // (external event-record nodes), so that the per-kernel device time of the
 // last replayed block can be read back.
@@ -541,6 +545,17 @@ int run_steps(qtb_ctx *c, int j0, int count, bool graph)
 {
     const MdLaunch &m = c->ml;
     const int obs = c->p.obs_stride;
+    if (c->d.n_ext_units) {
+        // external potentials, short rings: as many steps per launch as their records fit
+        // (n steps hold at most ceil(n / obs) records)
+        const int per = (int)std::min<long long>(count, (long long)c->ext_rows * obs);
+        for (int t = 0; t < count; t += per) {
+            const int n = std::min(per, count - t);
+            ProfMark pm(c, KC_FORCE);
+            launch_ext_steps(c->d, m, c->tabf, c->tab, j0 + t, n, (n + obs - 1) / obs, c->st);
+        }
+        if (!m.ext_long) return QTB_OK;
+    }
     for (int t = 0; t < count; ++t) {
         const int j = j0 + t, cur = j & 1;
         const bool keep = c->capturing;
@@ -1089,6 +1104,10 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
         S.icta0 = icta;
         icta += (h.N + integrate_atoms_per_cta(h.P, nm_big) - 1) / integrate_atoms_per_cta(h.P, nm_big);
         S.icta1 = icta;
+        S.eu0 = (int)c->ext_units.size();
+        if (!c->pair && h.P <= kExtMaxP)
+            for (int a = 0; a < h.N; a += kExtUnitAtoms) c->ext_units.push_back(make_int2(s, a));
+        S.eu1 = (int)c->ext_units.size();
         S.ccta0 = ccta;
         if (h.P > 1) ccta += (h.N + kCenAtoms - 1) / kCenAtoms;
         S.ccta1 = ccta;
@@ -1222,6 +1241,8 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
     m.n_icta = icta;
     m.n_ccta = ccta;
     m.n_ecta = ext_gx;
+    m.ext_long = 0;
+    for (int s = 0; s < n_sys; ++s) m.ext_long |= !c->pair && c->hs[s].P > kExtMaxP;
     m.nP = 0;
     for (int s = 0; s < n_sys; ++s) {
         bool seen = false;
@@ -1321,6 +1342,16 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
     cudaMemsetAsync(d.nrebuild, 0, sizeof(unsigned long long), c->st);
     cudaMemsetAsync(d.flag, 0, 2 * sizeof(unsigned), c->st);
     cudaMemsetAsync(d.gbar, 0, 2 * sizeof(unsigned), c->st);
+    d.ext_part = nullptr;
+    d.n_ext_units = (int)c->ext_units.size();
+    if (d.n_ext_units) {
+        // rows for as many records of a launch as fit kExtPartBytes (at least one)
+        c->ext_rows = (int)std::max<long long>(1, std::min<long long>(kBlockSteps / p->obs_stride + 1,
+                                                                      kExtPartBytes / (8LL * kExtRow * d.n_ext_units)));
+        d.ext_units = upload(c, c->ext_units);
+        d.ext_part = (double *)c->alloc(sizeof(double) * kExtRow * (size_t)d.n_ext_units * c->ext_rows);
+        if (!d.ext_units || !d.ext_part) return bail(fail(QTB_ERR_OOM, "device allocation failed"));
+    }
     d.eta = c->alloc(c->rsz * (size_t)kBlockSteps * (size_t)D);
     d.eta_blocks = 1;
     d.part = (double *)c->alloc(sizeof(double) * kNQ * (size_t)std::max(nforce, 1LL));

@@ -8,10 +8,12 @@ namespace qtb {
 
 // External separable potentials, one thread per bead-atom.  grid = (gx, nsys)
 template <class R>
-__global__ void __launch_bounds__(128) k_force_ext(Dev d, PairTabT<R> T, int kick)
+__global__ void __launch_bounds__(128) k_force_ext(Dev d, PairTabT<R> T, int kick, int j)
 {
     __shared__ double red[4][kNQ];
     const DSys S = d.sys[blockIdx.y];
+    if (kick && S.P <= kExtMaxP) return;  // stepped by k_ext_steps
+    const bool rec = !kick || (d.clock[0] * kBlockSteps + j + 1) % d.obs_stride == 0;
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     double acc[kNQ];
 #pragma unroll
@@ -44,6 +46,7 @@ __global__ void __launch_bounds__(128) k_force_ext(Dev d, PairTabT<R> T, int kic
                 v += hdtm * fb;
                 V[c * G + g] = v;
             }
+            if (!rec) continue;  // (the sums take the slow FP64 pipes)
             e += (double)ex;
             ke += 0.5 * T.mass_mvv[t] * (double)v * (double)v;
             x2 += (double)x * (double)x;
@@ -54,8 +57,10 @@ __global__ void __launch_bounds__(128) k_force_ext(Dev d, PairTabT<R> T, int kic
         acc[Q_V] = e;
         acc[Q_X2] = x2;
     }
+    if (!rec) return;
     for (int q = 0; q < kNQ; ++q) acc[q] = warp_sum(acc[q]);
-    cta_store_partials(acc, red, d.part + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kNQ);}
+    cta_store_partials(acc, red, d.part + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kNQ);
+}
 
 // ---------------------------------------------------------------------------
 // Per-system reduction into the observable record (external potentials).
@@ -65,7 +70,7 @@ __global__ void k_reduce(Dev d, int j, int record)
     __shared__ double sh[4][kNQ + 1];
     const long long step = d.clock[0] * kBlockSteps + j + 1;  // steps completed
     // during stepping only the recorded steps are reduced (record < 0: always)
-    if (record >= 0 && step % d.obs_stride != 0) return;
+    if (record >= 0 && (step % d.obs_stride != 0 || d.sys[blockIdx.x].P <= kExtMaxP)) return;
     reduce_system<false>(d, blockIdx.x, step, record, sh, d.part, d.sys[blockIdx.x].fcta0, d.sys[blockIdx.x].fcta1);
 }
 
@@ -107,6 +112,7 @@ __global__ void __launch_bounds__(32 * kCenWarps) k_centroid(Dev d, int j, int r
     if (record >= 0 && step % d.obs_stride != 0 && !d.npt) return;
     const int cta = blockIdx.x, s = d.ccta_sys[cta];
     const DSys S = d.sys[s];
+    if (PM == PM_FREE && record >= 0 && S.P <= kExtMaxP) return;  // recorded by k_ext_records
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int N = S.N, P = S.P;
     const int i = (cta - S.ccta0) * kCenAtoms + lane;
@@ -553,11 +559,13 @@ static cudaError_t nm_prepare(const MdLaunch &m)
 {
     for (int u = 0; u < m.nP; ++u) {
         cudaError_t e = cudaSuccess;
-        switch (m.Pvals[u]) {
-#define QTB_P(PP) case PP: e = nm_prepare_one<PP, PM, R>(m.nm_big); break;
-            QTB_P(2) QTB_P(3) QTB_P(4) QTB_P(5) QTB_P(6) QTB_P(8) QTB_P(16) QTB_P(32)
+        if (PM != PM_FREE || m.Pvals[u] > kExtMaxP) {
+            switch (m.Pvals[u]) {
+#define QTB_P(PP) case PP: if constexpr (PM != PM_FREE || PP > kExtMaxP) e = nm_prepare_one<PP, PM, R>(m.nm_big); break;
+                QTB_P(2) QTB_P(3) QTB_P(4) QTB_P(5) QTB_P(6) QTB_P(8) QTB_P(16) QTB_P(32)
 #undef QTB_P
-            default: break;
+                default: break;
+            }
         }
         if (e != cudaSuccess) return e;
     }
@@ -574,12 +582,17 @@ template <int PM, class R>
 static void integrate_all(const Dev &d, const MdLaunch &m, int j, int cur, cudaStream_t st)
 {
     for (int u = 0; u < m.nP; ++u) {
-        switch (m.Pvals[u]) {
-            case 1: pdl_launch(k_integrate<1, PM, R>, m.n_icta, 128, 0, st, d, j, cur); break;
+        if constexpr (PM == PM_FREE) {  // shorter rings: k_ext_steps
+            if (m.Pvals[u] == 16) nm_launch<16, PM, R>(d, m, j, cur, st);
+            else if (m.Pvals[u] == 32) nm_launch<32, PM, R>(d, m, j, cur, st);
+        } else {
+            switch (m.Pvals[u]) {
+                case 1: pdl_launch(k_integrate<1, PM, R>, m.n_icta, 128, 0, st, d, j, cur); break;
 #define QTB_P(PP) case PP: nm_launch<PP, PM, R>(d, m, j, cur, st); break;
-            QTB_P(2) QTB_P(3) QTB_P(4) QTB_P(5) QTB_P(6) QTB_P(8) QTB_P(16) QTB_P(32)
+                QTB_P(2) QTB_P(3) QTB_P(4) QTB_P(5) QTB_P(6) QTB_P(8) QTB_P(16) QTB_P(32)
 #undef QTB_P
-            default: break;
+                default: break;
+            }
         }
     }
 }
@@ -614,8 +627,8 @@ cudaError_t launch_force(const Dev &d, const MdLaunch &m, const PairTabT<float> 
         return step_force_l128(d, m, Tf, Td, kick, j, cur, adv, rec, st);
     }
     dim3 g((unsigned)m.n_ecta, (unsigned)d.nsys);
-    if (m.mixed) k_force_ext<float><<<g, 128, 0, st>>>(d, Tf, kick);
-    else k_force_ext<double><<<g, 128, 0, st>>>(d, Td, kick);
+    if (m.mixed) k_force_ext<float><<<g, 128, 0, st>>>(d, Tf, kick, j);
+    else k_force_ext<double><<<g, 128, 0, st>>>(d, Td, kick, j);
     return cudaGetLastError();
 }
 

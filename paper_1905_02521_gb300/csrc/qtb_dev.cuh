@@ -24,6 +24,8 @@ constexpr int kNQ = 16;              // partial sums per CTA (see Q_* below)
 constexpr int kRedGroup = 16;        // force units per group of the two-level record reduction
 constexpr int kFixBits = 30;         // fixed-point positions: box edge = 2^30 units
 constexpr int kMaxTypes = 4;
+constexpr int kExtMaxP = 8;          // external potentials: longest ring carried through many steps a launch
+constexpr int kExtRow = 16;          // doubles of a row of Dev::ext_part
 constexpr int kFitN = 10;            // coefficients of the FP32 Coulomb fits (degree 9)
 constexpr int kWarpsPerForceCta = 8;  // warps of the list build kernel
 
@@ -97,6 +99,7 @@ struct DSys {
     int icta0, icta1;  // integrator CTA range
     int fcta0, fcta1;  // force CTA range (pair potential: of the 16-lane units)
     int grp0, ngrp;    // its groups of kRedGroup force units (two-level record reduction)
+    int eu0, eu1;      // external-potential units (Dev::ext_units; empty for long rings)
     int ccta0, ccta1;  // centroid-estimator CTA range (empty for one bead)
     int cell0, cell1;  // cells of all its replicas (pair potential)
     int rot0;          // offset of this system's mode rotation table
@@ -179,7 +182,11 @@ struct Dev {
     const int2 *units, *units_rec;
     int nunits, nunits_rec;
     const int *icta_sys;  // [integrator CTAs] system of each CTA
-    const int *ext_cta_sys;
+    // external potentials, rings of up to kExtMaxP beads (ext.cu): units (system, first
+    // atom), and a row of kExtRow sums per unit and record of a launch
+    const int2 *ext_units;
+    int n_ext_units;
+    double *ext_part;
     // state
     void *x;              // positions, SoA [3][G] (double, int32 or R by mode)
     void *v;              // velocities [3][G] (R)

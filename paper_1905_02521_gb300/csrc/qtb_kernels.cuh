@@ -60,6 +60,7 @@ struct MdLaunch {
     int n_icta;           // integrator CTAs
     int n_ccta;           // centroid-estimator CTAs (0: no ring polymer)
     int n_ecta;           // external-force CTAs per system
+    int ext_long;         // some system with an external potential has more than kExtMaxP beads
     int nP;               // number of distinct bead counts
     int Pvals[8];         // distinct bead counts
     int fused;            // all systems one-bead with a pair potential: the step kernel
@@ -100,6 +101,11 @@ void launch_integrate(const Dev &d, const MdLaunch &m, int j, int cur, cudaStrea
 // be recorded, then the kernel also reduces the observables
 cudaError_t launch_force(const Dev &d, const MdLaunch &m, const PairTabT<float> &Tf, const PairTabT<double> &Td,
                          int kick, int j, int cur, int adv, int rec, cudaStream_t st);
+// ext.cu: steps j0 .. j0 + count - 1 of the current block for every system with an external
+// potential and at most kExtMaxP beads, with the records that fall into them (at most max_rec)
+constexpr int kExtUnitAtoms = 32;  // atoms of a unit
+void launch_ext_steps(const Dev &d, const MdLaunch &m, const PairTabT<float> &Tf, const PairTabT<double> &Td, int j0,
+                      int count, int max_rec, cudaStream_t st);
 void launch_reduce(const Dev &d, const MdLaunch &m, int j, int record, cudaStream_t st);
 // centroid-virial estimators of the ring-polymer systems (record slots 18, 19),
 // after the force launch of a step that may be recorded (record < 0: latest only)

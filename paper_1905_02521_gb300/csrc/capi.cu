@@ -742,12 +742,12 @@ int rebuild_filters(qtb_ctx *c)
         c->release(c->dS);
         c->d_taps64 = (double *)c->alloc(sizeof(double) * tot);
         c->d_taps32 = (float *)c->alloc(sizeof(float) * tot);
-        c->dS = (double *)c->alloc(sizeof(double) * tot);
+        c->dS = (double *)c->alloc(sizeof(double) * 2 * tot);  // spectra, then the cosine tables
         if (!c->d_taps64 || !c->d_taps32 || !c->dS) return fail(QTB_ERR_OOM, "taps allocation failed");
         c->taps_cap = tot;
     }
     CUDA_TRY(cudaMemcpyAsync(c->dspec, spec.data(), sizeof(DSpec) * ns, cudaMemcpyHostToDevice, c->st));
-    launch_spectrum_taps(c->dspec, ns, Kmax, c->dS, c->d_taps64, c->d_taps32, kappa_model_weights(c->kmodel), c->st);
+    launch_spectrum_taps(c->dspec, ns, Kmax, c->dS, c->dS + tot, c->d_taps64, c->d_taps32, kappa_model_weights(c->kmodel), c->st);
     CUDA_TRY(cudaGetLastError());
     // ring geometry
     const int Kb = (Kmax + kBlockSteps - 1) / kBlockSteps;

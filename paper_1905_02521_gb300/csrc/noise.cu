@@ -260,202 +260,400 @@ __global__ void k_spectrum(const DSpec *spec, double *S)
     S[sp.taps0 + j] = spectrum_value(sp, 2.0 * kPi * j / (L * sp.dt));
 }
 
-__global__ void k_taps(const DSpec *spec, const double *S, double *h64, float *h32)
+// sqrt(S_j) in place and the table cos(2 pi j/L), j = 0..K (the cosine transform's
+// square roots and cosines, once each instead of once per tap: K^2 of either took 2 ms
+// of the FP64 pipes at K = 1024, now 0.1 ms)
+__global__ void k_taps_table(const DSpec *spec, double *S, double *cs)
 {
     const DSpec sp = spec[blockIdx.y];
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j > sp.K) return;
+    S[sp.taps0 + j] = sqrt(S[sp.taps0 + j]);
+    cs[sp.taps0 + j] = cospi(2.0 * (double)j / (double)(2 * sp.K + 1));
+}
+
+__global__ void k_taps(const DSpec *spec, const double *S, const double *cs, double *h64, float *h32)
+{
+    const DSpec sp = spec[blockIdx.y];
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k > sp.K) return;
-    const int K = sp.K;
-    const long long L = 2 * K + 1;
-    const double *Sj = S + sp.taps0;
+    const int K = sp.K, L = 2 * K + 1;
+    const double *Sj = S + sp.taps0, *cj = cs + sp.taps0;
     double acc = 0.0;
+    int m = 0;  // j k mod L
     for (int j = 1; j <= K; ++j) {
-        long long m = ((long long)j * k) % L;
-        acc += sqrt(Sj[j]) * cospi(2.0 * (double)m / (double)L);
+        m += k;
+        if (m >= L) m -= L;
+        acc += Sj[j] * cj[min(m, L - m)];
     }
-    double h = (sqrt(Sj[0]) + 2.0 * acc) / (double)L;
+    const double h = (Sj[0] + 2.0 * acc) / (double)L;
     h64[sp.taps0 + k] = h;
     h32[sp.taps0 + k] = (float)h;
 }
 
 // ---------------------------------------------------------------------------
-// kappa_P solve (Eq. 10), FP64: dense collocation rows, normal equations,
-// blocked Cholesky (many CTAs), triangular solves (one CTA), one refinement step.
+// kappa_P solve (Eq. 10), FP64: collocation rows, normal equations, blocked Cholesky,
+// triangular solves, one refinement step.
+//
+// A row has 2 P nonzeros on its P curves y_k(y), and the curves run together at large y:
+// of the 32 x 32 tiles of A most are zero, and the normal matrix is dense only in its
+// leading part (columns up to asinh sqrt(4 P)) and narrow-banded beyond.  Everything
+// below works on tiles and skips the zero ones (what they would add is exactly zero):
+// flags per tile of A, and per tile row of the factor the first nonzero tile
+// (Cholesky keeps that envelope).  One solve (P = 8, n = 1024): 3.0 ms; with dense
+// normal equations, one-warp panels and unblocked triangular solves 17.5.
+constexpr int kCholNb = 32;
 
-// rows m < 2n-1; A is (2n-1) x n row-major, zeroed by the caller
-__global__ void k_kappa_rows(int P, int n, double ymax, double y0, double *A, double *b)
+static inline int kappa_words(int n) { return ((n + kCholNb - 1) / kCholNb + 31) / 32; }  // flag words per tile row of A
+// envelope of the factor: ints in row 0 of M from column 32 on (the strict upper triangle
+// of M is not used outside the diagonal tiles; one tile has no envelope)
+__device__ __forceinline__ int *kappa_env(double *M) { return reinterpret_cast<int *>(M + kCholNb); }
+__device__ __forceinline__ const int *kappa_env(const double *M) { return reinterpret_cast<const int *>(M + kCholNb); }
+
+struct KappaTerm {
+    double w, lam;  // weight; position in the interval, or (i < 0) the tail's value
+    int i;          // left node of the interval, -1: beyond the grid, -2: no term
+};
+__device__ __forceinline__ KappaTerm kappa_term(int P, int n, double ymax, double y0, double dts, int m, int k)
 {
-    int m = blockIdx.x * blockDim.x + threadIdx.x;
-    int rows = 2 * n - 1;
-    if (m >= rows) return;
-    double dts = asinh(ymax / y0) / (n - 1);
-    double y = y0 * sinh(0.5 * m * dts);
-    double rhs = fth_dev(sqrt((double)P) * y);
-    double *Ar = A + (size_t)m * n;
-    for (int k = 0; k < P; ++k) {
-        double sk = sinpi((double)k / P);
-        double ck = 4.0 * P * sk * sk;
-        double yk = sqrt(y * y + ck);
-        double w = (k == 0) ? 1.0 : ((y * y + ck) > 0.0 ? y * y / (y * y + ck) : 0.0);
-        if (w == 0.0) continue;
-        if (yk <= ymax) {
-            int i = (int)(asinh(yk / y0) / dts);
-            if (i > n - 2) i = n - 2;
-            double ya = y0 * sinh(i * dts), yb = y0 * sinh((i + 1) * dts);
-            double lam = (yk - ya) / (yb - ya);
-            Ar[i] += w * (1.0 - lam);
-            Ar[i + 1] += w * lam;
-        } else {
-            rhs -= w * kappa_tail_dev(P, yk);
-        }
+    const double y = y0 * sinh(0.5 * m * dts), sk = sinpi((double)k / P), ck = 4.0 * P * sk * sk, yk = sqrt(y * y + ck);
+    KappaTerm t;
+    t.w = (k == 0) ? 1.0 : ((y * y + ck) > 0.0 ? y * y / (y * y + ck) : 0.0);
+    t.lam = 0.0;
+    t.i = -2;
+    if (t.w == 0.0) return t;
+    if (yk <= ymax) {
+        t.i = min((int)(asinh(yk / y0) / dts), n - 2);
+        const double ya = y0 * sinh(t.i * dts), yb = y0 * sinh((t.i + 1) * dts);
+        t.lam = (yk - ya) / (yb - ya);
+    } else {
+        t.i = -1;
+        t.lam = kappa_tail_dev(P, yk);
     }
-    double sc = 1.0 / fth_dev(sqrt((double)P) * y);
-    for (int i = 0; i < n; ++i) Ar[i] *= sc;
-    b[m] = rhs * sc;
+    return t;
 }
 
-// M = A^T A (n x n), r = A^T b; 32x32 tiles, 256 threads (each 4 outputs)
-__global__ void k_kappa_normal(int rows, int n, const double *A, const double *b, double *M, double *r)
+// the terms of every row (their inverse hyperbolic functions are most of the work), one
+// thread each; grid = (ceil(rows / 128), P)
+__global__ void k_kappa_terms(int P, int n, double ymax, double y0, KappaTerm *t)
+{
+    const int m = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    if (m < 2 * n - 1) t[(size_t)m * P + k] = kappa_term(P, n, ymax, y0, asinh(ymax / y0) / (n - 1), m, k);
+}
+
+// rows m < 2n-1 from their terms (null: formed here), unscaled; A is (2n-1) x n row-major,
+// zeroed by the caller; b[m] and, for k_kappa_scale, sc[m] = 1/f
+__global__ void k_kappa_rows(int P, int n, double ymax, double y0, const KappaTerm *terms, double *A, double *b, double *sc)
+{
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= 2 * n - 1) return;
+    const double dts = asinh(ymax / y0) / (n - 1), y = y0 * sinh(0.5 * m * dts);
+    const double f = fth_dev(sqrt((double)P) * y);
+    double rhs = f;
+    double *Ar = A + (size_t)m * n;
+    for (int k = 0; k < P; ++k) {
+        const KappaTerm t = terms ? terms[(size_t)m * P + k] : kappa_term(P, n, ymax, y0, dts, m, k);
+        if (t.i >= 0) {
+            Ar[t.i] += t.w * (1.0 - t.lam);
+            Ar[t.i + 1] += t.w * t.lam;
+        } else if (t.i == -1) {
+            rhs -= t.w * t.lam;
+        }
+    }
+    sc[m] = 1.0 / f;
+    b[m] = rhs * (1.0 / f);
+}
+
+// rows times sc, and the flags of their nonzero tiles; one CTA of 256 per 32 rows
+__global__ void k_kappa_scale(int n, const double *sc, double *A, unsigned *nz, int words)
+{
+    const int m0 = blockIdx.x * kCholNb, rows = 2 * n - 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int ct = warp; ct * kCholNb < n; ct += 8) {
+        const int i = ct * kCholNb + lane;
+        bool any = false;
+        for (int q = 0; q < kCholNb; ++q) {
+            const int m = m0 + q;
+            if (m < rows && i < n) {
+                const double a = A[(size_t)m * n + i];
+                if (a != 0.0) {
+                    any = true;
+                    A[(size_t)m * n + i] = a * sc[m];
+                }
+            }
+        }
+        if (__any_sync(0xffffffffu, any) && lane == 0 && nz) atomicOr(&nz[blockIdx.x * words + (ct >> 5)], 1u << (ct & 31));
+    }
+}
+
+// envelope: first tile column tj with a nonzero tile (ti, tj) of M = A^T A, per tile
+// row; one CTA per ti, one thread per tile row of A
+__global__ void k_kappa_envelope(int n, const unsigned *nz, int words, double *M)
+{
+    __shared__ int first;
+    const int ti = blockIdx.x, nmt = (2 * n - 1 + kCholNb - 1) / kCholNb;
+    if (threadIdx.x == 0) first = nz ? ti : 0;
+    __syncthreads();
+    for (int mt = threadIdx.x; nz && mt < nmt; mt += blockDim.x)
+        if ((nz[mt * words + (ti >> 5)] >> (ti & 31)) & 1u)
+            for (int w = 0; w < words; ++w)
+                if (nz[mt * words + w]) {
+                    atomicMin(&first, 32 * w + __ffs(nz[mt * words + w]) - 1);
+                    break;
+                }
+    __syncthreads();
+    if (threadIdx.x == 0) kappa_env(M)[ti] = first;
+}
+
+// M = A^T A, lower triangle, over the tile rows of A that meet both tile columns;
+// blockIdx.x enumerates the tiles (ti >= tj); 256 threads, each 4 outputs
+__global__ void k_kappa_normal(int n, const double *A, const unsigned *nz, int words, double *M)
 {
     __shared__ double ta[32][33], tb[32][33];
-    int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
-    int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // ty in 0..7
+    int tj = blockIdx.x, ti = 0;
+    while (tj > ti) { tj -= ti + 1; ++ti; }
+    const int rows = 2 * n - 1, nmt = (rows + kCholNb - 1) / kCholNb;
+    const int i0 = ti * 32, j0 = tj * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // ty in 0..7
     double acc[4] = {0, 0, 0, 0};
-    for (int m0 = 0; m0 < rows; m0 += 32) {
+    for (int mt = 0; mt < nmt; ++mt) {
+        if (nz) {
+            const unsigned fi = nz[mt * words + (ti >> 5)] >> (ti & 31), fj = nz[mt * words + (tj >> 5)] >> (tj & 31);
+            if (!(fi & fj & 1u)) continue;  // uniform over the CTA
+        }
+        const int m0 = mt * kCholNb;
         for (int q = 0; q < 4; ++q) {
-            int mm = m0 + ty + 8 * q;
+            const int mm = m0 + ty + 8 * q;
             ta[ty + 8 * q][tx] = (mm < rows && i0 + tx < n) ? A[(size_t)mm * n + i0 + tx] : 0.0;
             tb[ty + 8 * q][tx] = (mm < rows && j0 + tx < n) ? A[(size_t)mm * n + j0 + tx] : 0.0;
         }
         __syncthreads();
+#pragma unroll 8
         for (int mm = 0; mm < 32; ++mm)
             for (int q = 0; q < 4; ++q) acc[q] += ta[mm][ty + 8 * q] * tb[mm][tx];
         __syncthreads();
     }
     for (int q = 0; q < 4; ++q) {
-        int i = i0 + ty + 8 * q, j = j0 + tx;
+        const int i = i0 + ty + 8 * q, j = j0 + tx;
         if (i < n && j < n) M[(size_t)i * n + j] = acc[q];
     }
-    if (blockIdx.x == 0) {
-        // r = A^T b for rows i0..i0+31
-        if (threadIdx.x < 32) {
-            int i = i0 + threadIdx.x;
-            if (i < n) {
-                double s = 0.0;
-                for (int mm = 0; mm < rows; ++mm) s += A[(size_t)mm * n + i] * b[mm];
-                r[i] = s;
+}
+
+// g = A^T s; one CTA of 8 warps per 32 columns, the warps' sums added in warp order
+__global__ void k_kappa_atv(int n, const double *A, const double *s, double *g)
+{
+    __shared__ double part[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane, rows = 2 * n - 1;
+    double acc = 0.0;
+    if (i < n) {
+#pragma unroll 8
+        for (int m = warp; m < rows; m += 8) acc += A[(size_t)m * n + i] * s[m];
+    }
+    part[warp][lane] = acc;
+    __syncthreads();
+    if (warp == 0 && i < n) {
+        for (int w = 1; w < 8; ++w) acc += part[w][lane];
+        g[i] = acc;
+    }
+}
+
+// Blocked right-looking Cholesky of the lower triangle of M (n x n, row-major), panels
+// of kCholNb columns, two launches a panel.  A warp's FP64 instruction holds its quarter
+// of the SM for ~64 cycles, so a 32 x 32 block is spread over four warps, a row over
+// four lanes (columns c = g mod 4); the diagonal block is eliminated without square
+// roots (they follow for all rows at once).  Every CTA that needs its factor forms it
+// again, which costs less than a launch in between.  (One warp with a row a lane took 85
+// us a panel.)  A non-positive pivot sets ERR_SOLVE (the solve then continues on a
+// placeholder pivot).
+constexpr int kCholThreads = 4 * kCholNb;
+
+// 1/v: two Newton steps from the FP32 value where that is in range, else the quotient
+__device__ __forceinline__ double fast_rcp(double v)
+{
+    if (!(v > 1e-30 && v < 1e30)) return 1.0 / v;
+    double y = (double)(1.0f / (float)v);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) y = fma(y, fma(-v, y, 1.0), y);
+    return y;
+}
+
+struct CholSmem {
+    double L[kCholNb][kCholNb + 1];  // L[c][r]: column c of the factor (r > c)
+    double rd[kCholNb];              // reciprocals of its diagonal
+    double col[2][kCholNb];
+};
+
+// factor of the block at (k0, k0) into B, by threads 0 .. kCholThreads - 1 of a CTA whose
+// threads all call it
+__device__ __forceinline__ void chol_factor32(int n, int k0, const double *M, CholSmem &B, unsigned *err)
+{
+    const int t = threadIdx.x, r = t >> 2, g = t & 3;
+    const bool mine = t < kCholThreads;
+    double a[kCholNb / 4];
+#pragma unroll
+    for (int q = 0; q < kCholNb / 4; ++q) {
+        const int c = 4 * q + g;
+        a[q] = mine && k0 + r < n && c <= r ? M[(size_t)(k0 + r) * n + k0 + c] : (c == r ? 1.0 : 0.0);
+    }
+#pragma unroll
+    for (int j = 0; j < kCholNb; ++j) {
+        double *col = B.col[j & 1];
+        if (mine && g == (j & 3)) col[r] = a[j / 4];
+        __syncthreads();
+        if (mine && r >= j) {
+            double v = col[j];
+            if (!(v > 0.0)) {
+                if (r == j && g == 0 && err) atomicOr(err, (unsigned)ERR_SOLVE);
+                v = 1e-300;
+            }
+            const double x = col[r];
+            if (g == 0) {
+                if (r == j) B.rd[j] = v;
+                else B.L[j][r] = x;
+            }
+            if (r > j) {
+                const double f = x * fast_rcp(v);
+#pragma unroll
+                for (int q = j / 4; q < kCholNb / 4; ++q)
+                    if (4 * q + g > j) a[q] = fma(-f, col[4 * q + g], a[q]);  // (columns past r stay unused)
             }
         }
     }
+    __syncthreads();
+    if (t < kCholNb) B.rd[t] = rsqrt(B.rd[t]);
+    __syncthreads();
+    if (mine)
+        for (int c = g; c < r; c += 4) B.L[c][r] *= B.rd[c];
+    __syncthreads();
 }
 
-// Blocked right-looking Cholesky of the lower triangle of M (n x n, row-major),
-// panels of kCholNb columns: for each panel k0 the diagonal block is factored
-// by one CTA (k_chol_diag), the rows below it are solved against that factor
-// (k_chol_panel, L21 = A21 L11^-T, one CTA per kCholNb rows), and the trailing
-// lower triangle is updated, A22 -= L21 L21^T, by one CTA per kCholNb x
-// kCholNb tile (k_chol_update).  Same arithmetic as the unblocked
-// factorisation up to the order of the sums; a non-positive pivot sets
-// ERR_SOLVE (the solve then continues on a placeholder pivot).
-constexpr int kCholNb = 32;
-
-__global__ void k_chol_diag(int n, int k0, double *M, unsigned *err)
+// rows r0 = k0 + 32 (1 + blockIdx.x) .. (+32) of the panel: X L11^T = A21
+__global__ void __launch_bounds__(kCholThreads) k_chol_panel(int n, int k0, double *M)
 {
-    __shared__ double a[kCholNb][kCholNb + 1];
-    const int nb = min(kCholNb, n - k0);
-    const int r = threadIdx.x / kCholNb, c = threadIdx.x % kCholNb;
-    const bool in = r < nb && c < nb && c <= r;
-    if (in) a[r][c] = M[(size_t)(k0 + r) * n + k0 + c];
-    __syncthreads();
-    for (int j = 0; j < nb; ++j) {
-        if (r == j && c == j) {
-            double v = a[j][j];
-            if (!(v > 0.0)) { atomicOr(err, (unsigned)ERR_SOLVE); v = 1e-300; }
-            a[j][j] = sqrt(v);
+    __shared__ CholSmem B;
+    const int ti = k0 / kCholNb + 1 + blockIdx.x;
+    if (kappa_env(M)[ti] > k0 / kCholNb) return;  // zero rows (uniform over the CTA)
+    chol_factor32(n, k0, M, B, nullptr);
+    const int t = threadIdx.x, g = t & 3, r = ti * kCholNb + (t >> 2);
+    double a[kCholNb / 4];
+#pragma unroll
+    for (int q = 0; q < kCholNb / 4; ++q) a[q] = r < n ? M[(size_t)r * n + k0 + 4 * q + g] : 0.0;
+#pragma unroll
+    for (int j = 0; j < kCholNb; ++j) {
+        const double x = __shfl_sync(0xffffffffu, a[j / 4], j & 3, 4) * B.rd[j];
+        if (g == (j & 3)) a[j / 4] = x;
+#pragma unroll
+        for (int q = j / 4; q < kCholNb / 4; ++q)
+            if (4 * q + g > j) a[q] = fma(-x, B.L[j][4 * q + g], a[q]);
+    }
+    if (r < n)
+#pragma unroll
+        for (int q = 0; q < kCholNb / 4; ++q) M[(size_t)r * n + k0 + 4 * q + g] = a[q];
+}
+
+// trailing update below the panel, blockIdx.x - 1 enumerating the tiles (ti >= tj) of the
+// trailing matrix; block 0 stores the diagonal block's factor (read unfactored by the
+// panel's CTAs before) the way the triangular solves take it: reciprocal diagonal rd,
+// below it L_ij rd_j, above it L_ji rd_j
+__global__ void __launch_bounds__(256) k_chol_update(int n, int k0, double *M, unsigned *err)
+{
+    __shared__ union {
+        CholSmem B;
+        double L[2][kCholNb][kCholNb + 1];
+    } sm;
+    if (blockIdx.x == 0) {
+        chol_factor32(n, k0, M, sm.B, err);
+        for (int e = threadIdx.x; e < kCholNb * kCholNb; e += blockDim.x) {
+            const int r = e / kCholNb, c = e % kCholNb;
+            if (k0 + r < n && k0 + c < n)
+                M[(size_t)(k0 + r) * n + k0 + c] = r == c ? sm.B.rd[r] : r > c ? sm.B.L[c][r] * sm.B.rd[c] : sm.B.L[r][c] * sm.B.rd[c];
         }
-        __syncthreads();
-        if (in && c == j && r > j) a[r][j] /= a[j][j];
-        __syncthreads();
-        if (in && c > j) a[r][c] -= a[r][j] * a[c][j];
-        __syncthreads();
+        return;
     }
-    if (in) M[(size_t)(k0 + r) * n + k0 + c] = a[r][c];
-}
-
-// rows r0 = k0 + nb + blockIdx.x kCholNb .. (+kCholNb) of the panel: X L11^T = A21
-__global__ void k_chol_panel(int n, int k0, double *M)
-{
-    __shared__ double L[kCholNb][kCholNb + 1], X[kCholNb][kCholNb + 1];
-    const int nb = min(kCholNb, n - k0);
-    const int r0 = k0 + nb + blockIdx.x * kCholNb;
-    const int r = threadIdx.x / kCholNb, c = threadIdx.x % kCholNb;
-    const bool row_in = r0 + r < n && c < nb;
-    L[r][c] = (r < nb && c <= r) ? M[(size_t)(k0 + r) * n + k0 + c] : 0.0;
-    X[r][c] = row_in ? M[(size_t)(r0 + r) * n + k0 + c] : 0.0;
-    __syncthreads();
-    for (int j = 0; j < nb; ++j) {
-        if (c == j) X[r][j] /= L[j][j];
-        __syncthreads();
-        if (c > j && c < nb) X[r][c] -= X[r][j] * L[c][j];
-        __syncthreads();
-    }
-    if (row_in) M[(size_t)(r0 + r) * n + k0 + c] = X[r][c];
-}
-
-// trailing update of the lower triangle below the panel; blockIdx.x enumerates the
-// tiles (ti >= tj) of the (n - k0 - nb)^2 trailing matrix in kCholNb blocks
-__global__ void k_chol_update(int n, int k0, double *M)
-{
-    __shared__ double Li[kCholNb][kCholNb + 1], Lj[kCholNb][kCholNb + 1];
-    const int nb = min(kCholNb, n - k0);
-    const int t0 = k0 + nb;
-    int t = blockIdx.x, ti = 0;
-    while (t > ti) { t -= ti + 1; ++ti; }  // tile (ti, tj = t), tj <= ti
-    const int tj = t;
-    const int ri0 = t0 + ti * kCholNb, rj0 = t0 + tj * kCholNb;
-    for (int e = threadIdx.x; e < kCholNb * kCholNb; e += blockDim.x) {
-        const int a = e / kCholNb, q = e % kCholNb;
-        Li[a][q] = (ri0 + a < n && q < nb) ? M[(size_t)(ri0 + a) * n + k0 + q] : 0.0;
-        Lj[a][q] = (rj0 + a < n && q < nb) ? M[(size_t)(rj0 + a) * n + k0 + q] : 0.0;
+    double (*Li)[kCholNb + 1] = sm.L[0], (*Lj)[kCholNb + 1] = sm.L[1];
+    int tj = blockIdx.x - 1, ti = 0;
+    while (tj > ti) { tj -= ti + 1; ++ti; }
+    const int kt = k0 / kCholNb;
+    ti += kt + 1;
+    tj += kt + 1;
+    if (kappa_env(M)[ti] > kt || kappa_env(M)[tj] > kt) return;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, ri0 = ti * kCholNb, rj0 = tj * kCholNb;
+    for (int q = ty; q < kCholNb; q += 8) {
+        Li[q][tx] = ri0 + q < n ? M[(size_t)(ri0 + q) * n + k0 + tx] : 0.0;
+        Lj[q][tx] = rj0 + q < n ? M[(size_t)(rj0 + q) * n + k0 + tx] : 0.0;
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < kCholNb * kCholNb; e += blockDim.x) {
-        const int a = e / kCholNb, b = e % kCholNb;
-        const int row = ri0 + a, col = rj0 + b;
-        if (row >= n || col > row) continue;
-        double acc = 0.0;
-        for (int q = 0; q < nb; ++q) acc += Li[a][q] * Lj[b][q];
-        M[(size_t)row * n + col] -= acc;
+    double acc[4] = {0, 0, 0, 0};
+#pragma unroll 8
+    for (int e = 0; e < kCholNb; ++e)
+        for (int q = 0; q < 4; ++q) acc[q] += Li[ty + 8 * q][e] * Lj[tx][e];
+    for (int q = 0; q < 4; ++q) {
+        const int i = ri0 + ty + 8 * q, j = rj0 + tx;
+        if (i < n && j <= i) M[(size_t)i * n + j] -= acc[q];
     }
 }
 
 static void chol_blocked(int n, double *M, unsigned *err, cudaStream_t st)
 {
     for (int k0 = 0; k0 < n; k0 += kCholNb) {
-        const int nb = std::min(kCholNb, n - k0), rest = n - k0 - nb;
-        k_chol_diag<<<1, kCholNb * kCholNb, 0, st>>>(n, k0, M, err);
-        if (rest <= 0) break;
-        const int nt = (rest + kCholNb - 1) / kCholNb;
-        k_chol_panel<<<nt, kCholNb * kCholNb, 0, st>>>(n, k0, M);
-        k_chol_update<<<nt * (nt + 1) / 2, 256, 0, st>>>(n, k0, M);
+        const int nt = std::max(0, (n - k0 - 1) / kCholNb);  // tile rows below
+        if (nt) k_chol_panel<<<nt, kCholThreads, 0, st>>>(n, k0, M);
+        k_chol_update<<<1 + nt * (nt + 1) / 2, 256, 0, st>>>(n, k0, M, err);
     }
 }
 
-// Solve L L^T x = r in place (x overwrites r); one CTA.
-__global__ void k_kappa_trsv(int n, const double *M, double *r)
+// Solve L L^T x = r in place (x overwrites r), one CTA of 16 warps, block by block: the
+// warps gather what the solved blocks contribute (a tile each, within the envelope),
+// warp 0 adds that up in warp order and solves the block's triangle, whose entries come
+// scaled (k_chol_update): a step of that chain is one broadcast and one multiply-add.
+constexpr int kTrsvWarps = 16;
+__global__ void __launch_bounds__(32 * kTrsvWarps) k_kappa_trsv(int n, const double *M, double *r)
 {
-    __shared__ double xj;
-    for (int j = 0; j < n; ++j) {  // forward: L y = r
-        if (threadIdx.x == 0) { xj = r[j] / M[(size_t)j * n + j]; r[j] = xj; }
-        __syncthreads();
-        for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) r[i] -= M[(size_t)i * n + j] * xj;
-        __syncthreads();
-    }
-    for (int j = n - 1; j >= 0; --j) {  // backward: L^T x = y
-        if (threadIdx.x == 0) { xj = r[j] / M[(size_t)j * n + j]; r[j] = xj; }
-        __syncthreads();
-        for (int i = threadIdx.x; i < j; i += blockDim.x) r[i] -= M[(size_t)j * n + i] * xj;
-        __syncthreads();
+    __shared__ double part[kTrsvWarps][kCholNb], D[kCholNb][kCholNb + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nt = (n + kCholNb - 1) / kCholNb;
+    const int *env = kappa_env(M);
+    for (int pass = 0; pass < 2; ++pass) {  // 0: L y = r, 1: L^T x = y
+        for (int s = 0; s < nt; ++s) {
+            const int kt = pass ? nt - 1 - s : s, k0 = kt * kCholNb;
+            for (int q = warp; q < kCholNb; q += kTrsvWarps)
+                D[q][lane] = (k0 + q < n && k0 + lane < n) ? M[(size_t)(k0 + q) * n + k0 + lane] : (q == lane ? 1.0 : 0.0);
+            double acc = 0.0;
+            const int t0 = pass ? kt + 1 : (nt > 1 ? env[kt] : 0), t1 = pass ? nt : kt;
+            if (pass == 0) {
+                const int row = k0 + lane;
+                for (int tj = t0 + warp; tj < t1; tj += kTrsvWarps)
+                    if (row < n) {
+                        const double *Lr = M + (size_t)row * n + tj * kCholNb;
+#pragma unroll 16
+                        for (int e = 0; e < kCholNb; ++e) acc = fma(Lr[e], r[tj * kCholNb + e], acc);
+                    }
+            } else {
+                const int col = k0 + lane;
+                for (int ti = t0 + warp; ti < t1; ti += kTrsvWarps)
+                    if (env[ti] <= kt && col < n) {
+                        const int e1 = min(kCholNb, n - ti * kCholNb);
+#pragma unroll 16
+                        for (int e = 0; e < e1; ++e) acc = fma(M[(size_t)(ti * kCholNb + e) * n + col], r[ti * kCholNb + e], acc);
+                    }
+            }
+            part[warp][lane] = acc;
+            __syncthreads();
+            if (warp == 0) {
+                double x = k0 + lane < n ? r[k0 + lane] : 0.0;
+                for (int w = 0; w < min(kTrsvWarps, t1 - t0); ++w) x -= part[w][lane];
+                double l[kCholNb];
+#pragma unroll
+                for (int j = 0; j < kCholNb; ++j) l[j] = (pass == 0 ? j < lane : j > lane) ? D[lane][j] : 0.0;
+                if (pass == 0) {
+#pragma unroll
+                    for (int j = 0; j < kCholNb; ++j) x = fma(-l[j], __shfl_sync(0xffffffffu, x, j), x);
+                } else {
+#pragma unroll
+                    for (int j = kCholNb - 1; j >= 0; --j) x = fma(-l[j], __shfl_sync(0xffffffffu, x, j), x);
+                }
+                if (k0 + lane < n) r[k0 + lane] = x * D[lane][lane];
+            }
+            __syncthreads();
+        }
     }
 }
 
@@ -472,19 +670,12 @@ __global__ void k_kappa_resid(int rows, int n, const double *A, const double *b,
     if (m >= rows) return;
     const double *Ar = A + (size_t)m * n;
     double acc = 0.0;
-    for (int i = lane; i < n; i += 32) acc += Ar[i] * x[i];
+    for (int i = lane; i < n; i += 32) {
+        const double a = Ar[i];
+        if (a != 0.0) acc += a * x[i];
+    }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) s[m] = b[m] - acc;
-}
-
-// g[i] = sum_m A[m,i] s[m]; one thread per column
-__global__ void k_kappa_atv(int rows, int n, const double *A, const double *s, double *g)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double acc = 0.0;
-    for (int m = 0; m < rows; ++m) acc += A[(size_t)m * n + i] * s[m];
-    g[i] = acc;
 }
 
 __global__ void k_kappa_add(int n, double *x, const double *d)
@@ -645,32 +836,43 @@ cudaError_t filter_simt_prepare(int Kmax)
                                 (int)(sm / 2 + 16));
 }
 
-void launch_spectrum_taps(const DSpec *spec, int nsys, int Kmax, double *S, double *h64, float *h32,
+void launch_spectrum_taps(const DSpec *spec, int nsys, int Kmax, double *S, double *cs, double *h64, float *h32,
                           const float *mlp_w, cudaStream_t st)
 {
     k_spectrum<<<dim3((Kmax + 1 + 255) / 256, nsys), 256, 0, st>>>(spec, S);
     if (mlp_w) launch_spectrum_mlp(spec, nsys, Kmax, S, mlp_w, st);
-    k_taps<<<dim3((Kmax + 1 + 127) / 128, nsys), 128, 0, st>>>(spec, S, h64, h32);
+    k_taps_table<<<dim3((Kmax + 1 + 127) / 128, nsys), 128, 0, st>>>(spec, S, cs);
+    k_taps<<<dim3((Kmax + 1 + 31) / 32, nsys), 32, 0, st>>>(spec, S, cs, h64, h32);
 }
 
 void launch_kappa_solve(int P, int n, double ymax, double y0, double *A, double *b, double *M, double *r,
                         double *work, unsigned *err, cudaStream_t st)
 {
-    int rows = 2 * n - 1;
+    const int rows = 2 * n - 1, nt = (n + kCholNb - 1) / kCholNb, nmt = (rows + kCholNb - 1) / kCholNb, words = kappa_words(n);
+    // scratch before the factorisation: the terms in M, the rows' scales and the tile flags in work
+    // (small grids: too many terms for M, formed row by row)
+    KappaTerm *terms = sizeof(KappaTerm) * (size_t)rows * P <= sizeof(double) * (size_t)n * n ? reinterpret_cast<KappaTerm *>(M) : nullptr;
+    double *sc = work;
+    // (nmt words <= 2 n ints up to n = 2^15; beyond, no tile is skipped)
+    unsigned *nz = n <= (1 << 15) ? reinterpret_cast<unsigned *>(work + rows) : nullptr;
     cudaMemsetAsync(A, 0, sizeof(double) * (size_t)rows * n, st);
-    k_kappa_rows<<<(rows + 127) / 128, 128, 0, st>>>(P, n, ymax, y0, A, b);
-    k_kappa_normal<<<dim3((n + 31) / 32, (n + 31) / 32), 256, 0, st>>>(rows, n, A, b, M, r);
+    if (terms) k_kappa_terms<<<dim3((rows + 127) / 128, P), 128, 0, st>>>(P, n, ymax, y0, terms);
+    k_kappa_rows<<<(rows + 31) / 32, 32, 0, st>>>(P, n, ymax, y0, terms, A, b, sc);
+    if (nz) cudaMemsetAsync(nz, 0, sizeof(unsigned) * (size_t)nmt * words, st);
+    k_kappa_scale<<<nmt, 256, 0, st>>>(n, sc, A, nz, words);
+    k_kappa_normal<<<nt * (nt + 1) / 2, 256, 0, st>>>(n, A, nz, words, M);
+    if (nt > 1) k_kappa_envelope<<<nt, 64, 0, st>>>(n, nz, words, M);
+    k_kappa_atv<<<nt, 256, 0, st>>>(n, A, b, r);
     chol_blocked(n, M, err, st);
-    k_kappa_trsv<<<1, 1024, 0, st>>>(n, M, r);
+    k_kappa_trsv<<<1, 32 * kTrsvWarps, 0, st>>>(n, M, r);
     double *s = work, *g = work + rows;
     for (int it = 0; it < kKappaRefine; ++it) {
         k_kappa_resid<<<(rows * 32 + 255) / 256, 256, 0, st>>>(rows, n, A, b, r, s);
-        k_kappa_atv<<<(n + 127) / 128, 128, 0, st>>>(rows, n, A, s, g);
-        k_kappa_trsv<<<1, 1024, 0, st>>>(n, M, g);
+        k_kappa_atv<<<nt, 256, 0, st>>>(n, A, s, g);
+        k_kappa_trsv<<<1, 32 * kTrsvWarps, 0, st>>>(n, M, g);
         k_kappa_add<<<(n + 255) / 256, 256, 0, st>>>(n, r, g);
     }
 }
-
 
 size_t fourier_smem(int n, int fp64) { return (size_t)2 * kSegPairs * 2 * n * (fp64 ? 8 : 4); }
 

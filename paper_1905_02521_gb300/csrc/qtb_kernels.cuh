@@ -34,7 +34,7 @@ cudaError_t filter_fft_prepare();
 void launch_fft_tables(const Dev &d, const double *taps64, void *tw, void *G, cudaStream_t st);
 void launch_white_fft(const Dev &d, int max_dofp, long long blk, cudaStream_t st);
 void launch_filter_fft(const Dev &d, int max_dofp, cudaStream_t st);
-void launch_spectrum_taps(const DSpec *spec, int nsys, int Kmax, double *S, double *h64, float *h32,
+void launch_spectrum_taps(const DSpec *spec, int nsys, int Kmax, double *S, double *cs, double *h64, float *h32,
                           const float *mlp_w, cudaStream_t st);
 
 // mlp.cu: spectrum S_j = kT f(y_j) ratio_model(y_j, P) W(w_j) for systems in the learned mode

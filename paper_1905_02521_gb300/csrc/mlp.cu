@@ -50,125 +50,212 @@ __device__ float mlp_forward(const float *w, float x1, float x2)
     return out;
 }
 
-// One CTA = 64 samples (one per thread): forward, backward, and the CTA's
-// gradient of sum_s scale (out_s - t_s)^2 into gpart[blockIdx.x][kNP].
-__global__ void __launch_bounds__(kSamplesPerCta) k_mlp_grad(const float *__restrict__ w, const float2 *__restrict__ x,
-                                                            const float *__restrict__ t, int n, float scale,
-                                                            float *gpart, float *lpart)
+// One CTA = 64 samples: forward, backward, and the CTA's gradient of sum_s scale
+// (out_s - t_s)^2 into gpart[blockIdx.x][kNP].  The three 64 x 64 x 64 products (layer 2
+// forward, its transpose backward, its weight gradient) are what the pass consists of:
+// 256 threads hold 4 x 4 tiles of them in registers, both factors read along rows of
+// shared memory (the activations and deltas are kept in both orders for that), so that
+// two 16-byte loads feed 16 multiply-adds.  (One sample per thread, a load per
+// multiply-add on two warps: 82 us for 12800 samples; this form 26, both cold.)
+constexpr int kGradThreads = 256;
+constexpr int kRow = 68;  // row of a 64 x 64 matrix in shared memory (16-byte aligned, spread over the banks)
+struct GradSmem {
+    float W2[kH][kH];                                       // [j][i]
+    float W2t[kH][kRow];                                    // [i][j]; then d3 h2 [s][j]
+    float H1t[kH][kRow];                                    // [i][s]; then dL/dz1 [s][i]
+    float H1[kH][kRow];                                     // [s][i]
+    float D2[kH][kRow], D2t[kH][kRow];                      // dL/dz2 [s][j], [j][s]
+    float w1[2 * kH], b1[kH], b2[kH], w3[kH], x[kSamplesPerCta][2], d3[kSamplesPerCta], red[kSamplesPerCta];
+};
+
+// acc[a][b] += sum_k A[k][a0 + a] B[k][b0 + b], k ascending
+template <int RA, int RB>
+__device__ __forceinline__ void tile_product(float (&acc)[4][4], const float (*A)[RA], const float (*B)[RB], int a0, int b0)
 {
-    extern __shared__ float sm[];
-    float *sw = sm;                        // kNP weights
-    float *sH1 = sw + kNP + 3;             // [64][65] activations of layer 1
-    float *sG1 = sH1 + 64 * 65;            // dsilu(z1)
-    float *sH2 = sG1 + 64 * 65;            // activations of layer 2
-    float *sD2 = sH2 + 64 * 65;            // dL/dz2
-    float *sD1 = sD2 + 64 * 65;            // dL/dz1
-    float *sX = sD1 + 64 * 65;             // [64][2]
-    float *sD3 = sX + 128;                 // [64]
-    const int s = threadIdx.x;
-    const int gidx = blockIdx.x * kSamplesPerCta + s;
-    for (int p = s; p < kNP; p += blockDim.x) sw[p] = w[p];
-    __syncthreads();
-    const bool valid = gidx < n;
-    const float2 xs = valid ? x[gidx] : make_float2(0.f, 0.f);
-    sX[2 * s] = xs.x;
-    sX[2 * s + 1] = xs.y;
-    for (int i = 0; i < kH; ++i) {
-        const float z = sw[oW1 + 2 * i] * xs.x + sw[oW1 + 2 * i + 1] * xs.y + sw[oB1 + i];
-        sH1[s * 65 + i] = silu(z);
-        sG1[s * 65 + i] = dsilu(z);
-    }
-    float out = sw[oB3];
-    for (int j = 0; j < kH; ++j) {
-        float z = sw[oB2 + j];
-        for (int i = 0; i < kH; ++i) z += sw[oW2 + j * kH + i] * sH1[s * 65 + i];
-        const float h = silu(z);
-        sH2[s * 65 + j] = h;
-        sD2[s * 65 + j] = dsilu(z);  // temporarily dsilu(z2)
-        out += sw[oW3 + j] * h;
-    }
-    const float r = valid ? out - t[gidx] : 0.0f;
-    const float d3 = 2.0f * scale * r;
-    sD3[s] = d3;
-    for (int j = 0; j < kH; ++j) sD2[s * 65 + j] *= d3 * sw[oW3 + j];
-    for (int i = 0; i < kH; ++i) {
-        float a = 0.0f;
-        for (int j = 0; j < kH; ++j) a += sD2[s * 65 + j] * sw[oW2 + j * kH + i];
-        sD1[s * 65 + i] = a * sG1[s * 65 + i];
-    }
-    // loss partial (fixed-order tree)
-    __shared__ float red[kSamplesPerCta];
-    red[s] = scale * r * r;
-    __syncthreads();
-    for (int o = kSamplesPerCta / 2; o > 0; o >>= 1) {
-        if (s < o) red[s] += red[s + o];
-        __syncthreads();
-    }
-    if (s == 0) lpart[blockIdx.x] = red[0];
-    // gradient partials: each thread owns parameters p = s, s + 64, ...
-    float *g = gpart + (size_t)blockIdx.x * kNP;
-    for (int p = s; p < kNP; p += blockDim.x) {
-        float acc = 0.0f;
-        if (p < oB1) {
-            const int i = p >> 1, k = p & 1;
-            for (int q = 0; q < kSamplesPerCta; ++q) acc += sD1[q * 65 + i] * sX[2 * q + k];
-        } else if (p < oW2) {
-            const int i = p - oB1;
-            for (int q = 0; q < kSamplesPerCta; ++q) acc += sD1[q * 65 + i];
-        } else if (p < oB2) {
-            const int j = (p - oW2) / kH, i = (p - oW2) % kH;
-            for (int q = 0; q < kSamplesPerCta; ++q) acc += sD2[q * 65 + j] * sH1[q * 65 + i];
-        } else if (p < oW3) {
-            const int j = p - oB2;
-            for (int q = 0; q < kSamplesPerCta; ++q) acc += sD2[q * 65 + j];
-        } else if (p < oB3) {
-            const int j = p - oW3;
-            for (int q = 0; q < kSamplesPerCta; ++q) acc += sD3[q] * sH2[q * 65 + j];
-        } else {
-            for (int q = 0; q < kSamplesPerCta; ++q) acc += sD3[q];
-        }
-        g[p] = acc;
+#pragma unroll 8
+    for (int k = 0; k < kH; ++k) {
+        const float4 a = *reinterpret_cast<const float4 *>(&A[k][a0]), b = *reinterpret_cast<const float4 *>(&B[k][b0]);
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(av[p], bv[q], acc[p][q]);
     }
 }
 
-size_t mlp_grad_smem() { return sizeof(float) * (kNP + 3 + 5 * 64 * 65 + 128 + 64); }
+__global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float *__restrict__ w, const float2 *__restrict__ x,
+                                                           const float *__restrict__ t, int n, float scale, float *gpart,
+                                                           float *lpart)
+{
+    extern __shared__ __align__(16) unsigned char msm[];
+    GradSmem &S = *reinterpret_cast<GradSmem *>(msm);
+    const int tid = threadIdx.x;
+    for (int e = tid; e < kH * kH; e += kGradThreads) {
+        const float v = w[oW2 + e];
+        S.W2[e / kH][e % kH] = v;
+        S.W2t[e % kH][e / kH] = v;
+    }
+    if (tid < 2 * kH) S.w1[tid] = w[oW1 + tid];
+    if (tid < kH) {
+        S.b1[tid] = w[oB1 + tid];
+        S.b2[tid] = w[oB2 + tid];
+        S.w3[tid] = w[oW3 + tid];
+        const int gi = blockIdx.x * kSamplesPerCta + tid;
+        const float2 xs = gi < n ? x[gi] : make_float2(0.f, 0.f);
+        S.x[tid][0] = xs.x;
+        S.x[tid][1] = xs.y;
+    }
+    __syncthreads();
+    auto z1 = [&](int s, int i) { return S.w1[2 * i] * S.x[s][0] + S.w1[2 * i + 1] * S.x[s][1] + S.b1[i]; };
+    {   // layer 1: 16 units of one sample per thread
+        const int s = tid & 63, i0 = (tid >> 6) * 16;
+#pragma unroll
+        for (int k = 0; k < 16; k += 4) {
+            float h[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                h[q] = silu(z1(s, i0 + k + q));
+                S.H1t[i0 + k + q][s] = h[q];
+            }
+            *reinterpret_cast<float4 *>(&S.H1[s][i0 + k]) = make_float4(h[0], h[1], h[2], h[3]);
+        }
+    }
+    __syncthreads();
+    const int a0 = 4 * (tid >> 4), b0 = 4 * (tid & 15);  // tile: rows a0, columns b0
+    float acc[4][4], pr[4][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = S.b2[b0 + q];
+    tile_product(acc, S.H1t, S.W2t, a0, b0);  // z2[s][j]
+    // out_s over the 16 threads of a sample's row of tiles, deltas of layer 2
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const int s = a0 + p, gi = blockIdx.x * kSamplesPerCta + s;
+        float o = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            pr[p][q] = silu(acc[p][q]);
+            o = fmaf(S.w3[b0 + q], pr[p][q], o);
+        }
+#pragma unroll
+        for (int m = 8; m > 0; m >>= 1) o += __shfl_xor_sync(0xffffffffu, o, m);
+        const float r = gi < n ? o + w[oB3] - t[gi] : 0.0f, d3 = 2.0f * scale * r;
+        if ((tid & 15) == 0) {
+            S.d3[s] = d3;
+            S.red[s] = scale * r * r;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float d = dsilu(acc[p][q]) * (d3 * S.w3[b0 + q]);
+            acc[p][q] = d;
+            S.D2t[b0 + q][s] = d;
+            pr[p][q] *= d3;
+        }
+        *reinterpret_cast<float4 *>(&S.D2[s][b0]) = make_float4(acc[p][0], acc[p][1], acc[p][2], acc[p][3]);
+    }
+    __syncthreads();  // (every thread is done with W2t and H1t too)
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+        *reinterpret_cast<float4 *>(&S.W2t[a0 + p][b0]) = make_float4(pr[p][0], pr[p][1], pr[p][2], pr[p][3]);
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = 0.0f;
+    tile_product(acc, S.D2t, S.W2, a0, b0);  // dL/dh1[s][i]
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] *= dsilu(z1(a0 + p, b0 + q));
+        *reinterpret_cast<float4 *>(&S.H1t[a0 + p][b0]) = make_float4(acc[p][0], acc[p][1], acc[p][2], acc[p][3]);
+    }
+    float *g = gpart + (size_t)blockIdx.x * kNP;
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = 0.0f;
+    tile_product(acc, S.D2, S.H1, a0, b0);  // dL/dW2[j][i]
+#pragma unroll
+    for (int p = 0; p < 4; ++p)  // (a parameter row starts at an odd word: scalar stores)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) g[oW2 + (a0 + p) * kH + b0 + q] = acc[p][q];
+    __syncthreads();
+    // the vectors: a column sum over the samples each
+    {
+        const int c = tid & 63, what = tid >> 6;  // 0, 1: W1 columns, 2: b1 and b2, 3: W3 (and b3, the loss)
+        float u = 0.0f, v = 0.0f;
+        if (what < 2) {
+            for (int s = 0; s < kSamplesPerCta; ++s) u = fmaf(S.H1t[s][c], S.x[s][what], u);
+            g[oW1 + 2 * c + what] = u;
+        } else if (what == 2) {
+            for (int s = 0; s < kSamplesPerCta; ++s) {
+                u += S.H1t[s][c];
+                v += S.D2[s][c];
+            }
+            g[oB1 + c] = u;
+            g[oB2 + c] = v;
+        } else {
+            for (int s = 0; s < kSamplesPerCta; ++s) u += S.W2t[s][c];
+            g[oW3 + c] = u;
+            if (c < 2) {
+                const float *src = c ? S.red : S.d3;
+                for (int s = 0; s < kSamplesPerCta; ++s) v += src[s];
+                if (c) lpart[blockIdx.x] = v;
+                else g[oB3] = v;
+            }
+        }
+    }
+}
+
+size_t mlp_grad_smem() { return sizeof(GradSmem); }
 
 struct AdamState {
     int iter;  // Adam step count so far
 };
 
-// Sum the CTA partials in fixed order; optionally take one Adam step.
-// One thread per parameter.  lr_sched: lr0 * decay^(iter / iters)
-__global__ void k_mlp_reduce_adam(const float *gpart, int nblk, float *w, float *m, float *v, float *gout,
-                                  const float *lpart, float *loss_out, AdamState *st, float lr0, float decay,
-                                  int iters, int update)
+// Sum the CTA partials in a fixed order (a warp an eighth of them, then the warps);
+// optionally take one Adam step, number st->iter + ahead.  A CTA per 32 parameters.
+// lr_sched: lr0 * decay^(iter / iters)
+__global__ void __launch_bounds__(256) k_mlp_reduce_adam(const float *gpart, int nblk, float *w, float *m, float *v,
+                                                         float *gout, const float *lpart, float *loss_out,
+                                                         const AdamState *st, int ahead, float lr0, float decay, int iters,
+                                                         int update)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int it = st->iter;
+    __shared__ float part[8][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
+    float g = 0.0f;
     if (p < kNP) {
-        float g = 0.0f;
-        for (int b = 0; b < nblk; ++b) g += gpart[(size_t)b * kNP + p];
-        if (gout) gout[p] = g;
-        if (update) {
-            const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-            const float mm = b1 * m[p] + (1.0f - b1) * g;
-            const float vv = b2 * v[p] + (1.0f - b2) * g * g;
-            m[p] = mm;
-            v[p] = vv;
-            const float tt = (float)(it + 1);
-            const float lr = lr0 * powf(decay, (float)it / (float)iters);
-            const float mh = mm / (1.0f - powf(b1, tt)), vh = vv / (1.0f - powf(b2, tt));
-            w[p] -= lr * mh / (sqrtf(vh) + eps);
-        }
+#pragma unroll 8
+        for (int b = warp; b < nblk; b += 8) g += gpart[(size_t)b * kNP + p];
     }
-    if (p == 0 && loss_out) {
+    part[warp][lane] = g;
+    if (blockIdx.x == gridDim.x - 1 && loss_out && warp == 7) {
         float l = 0.0f;
-        for (int b = 0; b < nblk; ++b) l += lpart[b];
-        *loss_out = l;
+        for (int b = lane; b < nblk; b += 32) l += lpart[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) *loss_out = l;
+    }
+    __syncthreads();
+    if (warp != 0 || p >= kNP) return;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) g += part[k][lane];
+    if (gout) gout[p] = g;
+    if (update) {
+        const int it = st->iter + ahead;
+        const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+        const float mm = b1 * m[p] + (1.0f - b1) * g;
+        const float vv = b2 * v[p] + (1.0f - b2) * g * g;
+        m[p] = mm;
+        v[p] = vv;
+        const float tt = (float)(it + 1);
+        const float lr = lr0 * powf(decay, (float)it / (float)iters);
+        const float mh = mm / (1.0f - powf(b1, tt)), vh = vv / (1.0f - powf(b2, tt));
+        w[p] -= lr * mh / (sqrtf(vh) + eps);
     }
 }
 
-__global__ void k_mlp_tick(AdamState *st) { st->iter += 1; }
+__global__ void k_mlp_tick(AdamState *st, int steps) { st->iter += steps; }
 
 // ratio kappa_P/theta at n points
 __global__ void k_mlp_infer(const float *w, const float2 *x, int n, float *out)
@@ -315,9 +402,9 @@ int qtb_kappa_model_grad(qtb_kappa_model *M, const float *x, const float *t, int
     cudaMemcpy(dx, x, sizeof(float) * 2 * n, cudaMemcpyHostToDevice);
     cudaMemcpy(dt, t, sizeof(float) * n, cudaMemcpyHostToDevice);
     cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_grad_smem());
-    k_mlp_grad<<<nblk, kSamplesPerCta, mlp_grad_smem()>>>(M->w, reinterpret_cast<const float2 *>(dx), dt, n,
-                                                          1.0f / n, gp, lp);
-    k_mlp_reduce_adam<<<(kNP + 255) / 256, 256>>>(gp, nblk, M->w, M->m, M->v, gd, lp, ld, st, 0.f, 1.f, 1, 0);
+    k_mlp_grad<<<nblk, kGradThreads, mlp_grad_smem()>>>(M->w, reinterpret_cast<const float2 *>(dx), dt, n,
+                                                        1.0f / n, gp, lp);
+    k_mlp_reduce_adam<<<(kNP + 31) / 32, 256>>>(gp, nblk, M->w, M->m, M->v, gd, lp, ld, st, 0, 0.f, 1.f, 1, 0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpy(grad, gd, sizeof(float) * kNP, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess && loss) e = cudaMemcpy(loss, ld, sizeof(float), cudaMemcpyDeviceToHost);
@@ -387,12 +474,12 @@ int qtb_kappa_model_train(qtb_kappa_model *M, const int *P_list, int nP, int n_p
     cudaGraphExec_t ge = nullptr;
     cudaStreamBeginCapture(sm, cudaStreamCaptureModeThreadLocal);
     for (int it = 0; it < per_graph; ++it) {
-        k_mlp_grad<<<nblk, kSamplesPerCta, mlp_grad_smem(), sm>>>(M->w, reinterpret_cast<const float2 *>(dx), dt, n,
-                                                                  1.0f / n, gp, lp);
-        k_mlp_reduce_adam<<<(kNP + 255) / 256, 256, 0, sm>>>(gp, nblk, M->w, M->m, M->v, nullptr, lp, ld, st, 3e-3f,
-                                                             3e-3f, iters, 1);
-        k_mlp_tick<<<1, 1, 0, sm>>>(st);
+        k_mlp_grad<<<nblk, kGradThreads, mlp_grad_smem(), sm>>>(M->w, reinterpret_cast<const float2 *>(dx), dt, n,
+                                                                1.0f / n, gp, lp);
+        k_mlp_reduce_adam<<<(kNP + 31) / 32, 256, 0, sm>>>(gp, nblk, M->w, M->m, M->v, nullptr, lp, ld, st, it, 3e-3f,
+                                                           3e-3f, iters, 1);
     }
+    k_mlp_tick<<<1, 1, 0, sm>>>(st, per_graph);
     cudaError_t e = cudaStreamEndCapture(sm, &g);
     if (e == cudaSuccess) e = cudaGraphInstantiate(&ge, g, 0);
     if (e == cudaSuccess) {

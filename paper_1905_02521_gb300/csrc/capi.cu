@@ -220,56 +220,104 @@ void fit_erfcx(double xmax, double c[12])
         for (int j = 0; j < n; ++j) c[j] += a[k] * Tm[k][j];
 }
 
-// The damped Coulomb terms of the FP32 step kernel (pair_poly) as polynomials in
-// u = 2 r^2/rc^2 - 1: cf fits -al^3 (erf x - 2 x e^{-x^2}/sqrt(pi))/x^3 and ce fits
-// al erf(x)/x, x = al r (Chebyshev interpolation, converted to monomials).  False
-// when an error exceeds 1e-8 of 1/r^3 (cf) or 1/r (ce) at the cutoff: a sixth of an
-// FP32 rounding of the term they are taken from.
-bool fit_coulomb(double al, double rc, double *cf, double *ce)
+// Double-double arithmetic (Dekker, Knuth) for the fits of the pair terms, whose
+// coefficients shall carry no error but their own rounding.
+struct Dd {
+    double h, l;
+};
+Dd dd_sum(double a, double b)
 {
-    const int n = kFitN;
-    auto f = [&](int which, double r) {
-        const double x = al * r, x2 = x * x;
-        double s;
-        if (x < 0.5) {  // power series in x^2
-            double t = 1.0;
-            s = 0.0;
-            for (int k = 0; k < 16; ++k) {
-                s += t * (which ? 1.0 / (2 * k + 1) : 2.0 / (2 * k + 3));
-                t *= -x2 / (k + 1);
-            }
-            s *= 2.0 / std::sqrt(kPi);
-        } else {
-            s = which ? std::erf(x) / x : (std::erf(x) - 2.0 * x / std::sqrt(kPi) * std::exp(-x2)) / (x2 * x);
+    const double s = a + b, t = s - a;
+    return {s, (a - (s - t)) + (b - t)};
+}
+Dd operator+(Dd a, Dd b)
+{
+    const Dd s = dd_sum(a.h, b.h);
+    return dd_sum(s.h, s.l + (a.l + b.l));
+}
+Dd operator-(Dd a) { return {-a.h, -a.l}; }
+Dd operator*(Dd a, Dd b)
+{
+    const double p = a.h * b.h;
+    return dd_sum(p, std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+Dd operator/(Dd a, Dd b)
+{
+    const double q = a.h / b.h;
+    const Dd r = a + -(Dd{q, 0.0} * b);
+    return dd_sum(q, (r.h + r.l) / b.h);
+}
+
+// Interpolant of f on [-1, 1] at n (<= 16) nodes near the Chebyshev points, as monomial
+// coefficients: Newton's divided differences, expanded.  lo: what the rounding of the first
+// two dropped.
+template <class F> void fit_poly(int n, double *c, double *lo, F f)
+{
+    double u[16];
+    Dd d[16], m[16];
+    for (int i = 0; i < n; ++i) {
+        u[i] = std::cos(kPi * (2 * i + 1) / (2 * n));
+        d[i] = f(u[i]);
+    }
+    for (int k = 1; k < n; ++k)
+        for (int i = n - 1; i >= k; --i) d[i] = (d[i] + -d[i - 1]) / dd_sum(u[i], -u[i - k]);
+    for (int k = 0; k < n; ++k) m[k] = {0.0, 0.0};
+    for (int i = n - 1; i >= 0; --i) {  // m <- m (u - u_i) + d_i
+        for (int k = n - 1; k > 0; --k) m[k] = m[k - 1] + -(m[k] * Dd{u[i], 0.0});
+        m[0] = d[i] + -(m[0] * Dd{u[i], 0.0});
+    }
+    for (int k = 0; k < n; ++k) c[k] = m[k].h;
+    lo[0] = m[0].l;
+    lo[1] = m[1].l;
+}
+
+// The damped Coulomb terms of the step kernel (pair_poly) as polynomials of n
+// coefficients in u = 2 r^2/rc^2 - 1: cf fits -al^3 (erf x - 2 x e^{-x^2}/sqrt(pi))/x^3
+// and ce fits al erf(x)/x, x = al r, from their power series in x^2.  False when an
+// error exceeds tol of 1/r^3 (cf) or 1/r (ce) at the cutoff (FP32: 1e-8, a sixth of a
+// rounding of the term they are taken from; FP64: 5e-16) or the series would lose digits.
+bool fit_coulomb(double al, double rc, int n, double tol, double *cf, double *ce, double *ce_lo)
+{
+    const Dd two_sqrtpi = {1.1283791670955126, 1.533545961316588e-17}, a1 = {al, 0.0};
+    if (!(al * rc < 4.0)) return false;
+    auto f = [&](int which, double u) {
+        const Dd x2 = a1 * a1 * Dd{rc, 0.0} * Dd{rc, 0.0} * (dd_sum(u, 1.0) * Dd{0.5, 0.0});
+        Dd t = {1.0, 0.0}, s = {0.0, 0.0};
+        for (int k = 0; k < 120 && std::fabs(t.h) > 1e-36; ++k) {  // (-x^2)^k/k! over 2k+1 (ce), half of 2k+3 (cf)
+            s = s + t * (which ? Dd{1.0, 0.0} / Dd{2.0 * k + 1.0, 0.0} : Dd{2.0, 0.0} / Dd{2.0 * k + 3.0, 0.0});
+            t = -(t * x2) / Dd{k + 1.0, 0.0};
         }
-        return which ? al * s : -al * al * al * s;
+        s = s * two_sqrtpi * a1;
+        return which ? s : -(s * a1 * a1);
     };
-    double Tm[kFitN][kFitN] = {{0}};
-    Tm[0][0] = 1.0;
-    Tm[1][1] = 1.0;
-    for (int k = 2; k < n; ++k)
-        for (int j = 0; j < n; ++j) Tm[k][j] = (j > 0 ? 2.0 * Tm[k - 1][j - 1] : 0.0) - Tm[k - 2][j];
     bool ok = true;
     for (int w = 0; w < 2; ++w) {
         double *c = w ? ce : cf;
-        for (int k = 0; k < n; ++k) c[k] = 0.0;
-        for (int k = 0; k < n; ++k) {
-            double a = 0.0;
-            for (int i = 0; i < n; ++i) {
-                const double th = kPi * (i + 0.5) / n;
-                a += f(w, rc * std::sqrt(0.5 * (std::cos(th) + 1.0))) * std::cos(k * th);
-            }
-            a *= (k ? 2.0 : 1.0) / n;
-            for (int j = 0; j < n; ++j) c[j] += a * Tm[k][j];
-        }
-        for (int i = 0; i <= 400; ++i) {
-            const double u = -1.0 + i / 200.0, r = rc * std::sqrt(0.5 * (u + 1.0));
-            double p = 0.0;
-            for (int k = n - 1; k >= 0; --k) p = p * u + c[k];
-            if (!(std::fabs(p - f(w, r)) * (w ? rc : rc * rc * rc) <= 1e-8)) ok = false;
+        fit_poly(n, c, ce_lo, [&](double u) { return f(w, u); });  // (ce is the last)
+        for (int i = 0; i <= 100; ++i) {
+            const double u = -1.0 + i / 50.0;
+            Dd p = {0.0, 0.0};
+            for (int k = n - 1; k >= 0; --k) p = p * Dd{u, 0.0} + Dd{c[k], 0.0};
+            if (!(std::fabs((p + -f(w, u)).h) * (w ? rc : rc * rc * rc) <= tol)) ok = false;
         }
     }
     return ok;
+}
+
+// 2^f on |f| <= 1/2, n coefficients (power series of exp(f ln 2))
+void fit_exp2(int n, double *c)
+{
+    const Dd ln2 = {0.6931471805599453, 2.3190468138462996e-17};
+    double lo[2];
+    fit_poly(n, c, lo, [&](double u) {  // u = 2 f
+        Dd t = {1.0, 0.0}, s = {0.0, 0.0};
+        for (int k = 1; k < 40; ++k) {
+            s = s + t;
+            t = t * ln2 * Dd{0.5 * u, 0.0} / Dd{(double)k, 0.0};
+        }
+        return s;
+    });
+    for (int k = 0; k < n; ++k) c[k] = std::ldexp(c[k], k);
 }
 
 static int decode_err_word(qtb_ctx *c, unsigned e);
@@ -848,11 +896,12 @@ double effective_skin(const qtb_params *p, double T)
 // 8000: 15.1 / 10.7 / 14.7, 10648: 14.4 / 16.9 / 17.9, 32768: 36.9 / 32.0, 64000: 62.4 /
 // 62.8; ring polymers (7 CTAs per SM) 1728: 10.8 / 9.7 / 9.3, 4096: 13.9 / 13.4 / 14.9,
 // 55296: 76.4 / 70.7, 221184: 231 / 236, 864000: 887 / 917; FP64 form (bound by the
-// FP64 pipes, so its work is spread over the SMs) 64: 219 / 116 / 73 / 32, 512: 203 / 112 /
-// 83 / 61, 1728: 276 / 229 / 194 / 159, 4096: 630 / 369 / 385 / 364.
+// FP64 pipes, so its work is spread over the SMs) 64: 103 / 58 / 38 / 20, 512: 92 / 51 /
+// 39 / 29, 1728: 123 / 103 / 89 / 77, 2744: 200 / 163 / 175 / 123, 4096: 278 / 164 / 176 /
+// 172, 8000: 326 / 324 / 347 / 324.
 int default_lanes(long long n, bool fp64, bool one_bead, int nsm)
 {
-    if (fp64) return n <= 27LL * nsm ? 128 : 16;
+    if (fp64) return n <= 24LL * nsm ? 128 : 16;
     if (!one_bead) return n <= 14LL * nsm ? 32 : n <= 1024LL * nsm ? 16 : 8;
     if (n <= 2LL * nsm) return 128;
     if (n <= 28LL * nsm) return 32;                     // one wave: 7 CTAs of 4 bead-atoms per SM
@@ -1009,16 +1058,29 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
         double cfit[12];
         fit_erfcx(xmax, cfit);
         for (int k = 0; k < 12; ++k) F.erfc_c[k] = (float)cfit[k];
-        double cf[kFitN], ce[kFitN];
-        poly_ok = c->pair && T.alpha >= 0.0 && fit_coulomb(T.alpha, T.rc, cf, ce);
+        double cf[kFitN<float>], ce[kFitN<float>], lo[2];
+        poly_ok = c->pair && c->mixed && T.alpha >= 0.0 && fit_coulomb(T.alpha, T.rc, kFitN<float>, 1e-8, cf, ce, lo);
         if (poly_ok) {
             F.r2_us = (float)(2.0 / T.rc2);
-            for (int k = 0; k < kFitN; ++k) {
+            for (int k = 0; k < kFitN<float>; ++k) {
                 F.cf[k] = (float)cf[k];
                 F.ce[k] = (float)ce[k];
             }
         }
         for (int t = 0; t < NT; ++t) F.nl2e_rho[t] = (float)(-log2e * T.inv_rho[t]);
+        if (c->pair && !c->mixed) {
+            poly_ok = T.alpha >= 0.0 && fit_coulomb(T.alpha, T.rc, kFitN<double>, 5e-16, T.cf, T.ce, T.ce_lo);
+            T.r2_us = 2.0 / T.rc2;
+            for (int t = 0; t < NT; ++t) {
+                // -log2(e)/rho in two words, log2(e) too
+                const double rho = T.inv_rho[t] != 0.0 ? p->buck_rho[(t / kMaxTypes) * nt + t % kMaxTypes] : 0.0;
+                const double hi = -log2e * T.inv_rho[t];
+                T.nl2e_rho[t] = hi;
+                // the residual of hi rho = -(log2e + 2.0355273740931033e-17)
+                T.nl2e_lo[t] = rho != 0.0 ? (-std::fma(hi, rho, log2e) - 2.0355273740931033e-17) / rho : 0.0;
+            }
+            fit_exp2(kExpN, T.ex2c);
+        }
     }
 
     // ---- layout
@@ -1188,7 +1250,7 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
     // minimum image suffices for the list entries when every edge exceeds twice the
     // largest separation an entry can reach before a rebuild (r_cut + skin, plus skin/2
     // of motion for each of the two atoms); not with a changing cell.
-    c->ml.variant = (c->pair && c->mixed && poly_ok) ? (p->npt ? 1 : 2) : 0;
+    c->ml.variant = !(c->pair && poly_ok) ? 0 : (p->npt || !c->mixed) ? 1 : 2;
     for (int s = 0; s < n_sys && c->ml.variant == 2; ++s)
         for (int k = 0; k < 3; ++k)
             if (!(sys[s].box[k] > 2.0 * (p->r_cut + 2.0 * c->skins[s]))) c->ml.variant = 1;

@@ -673,7 +673,7 @@ __device__ __forceinline__ double my_sqrt(double x) { return sqrt(x); }
 // Coefficients of one type pair, staged in shared memory by the step kernel
 // (the pair type varies across the lanes of a warp).
 template <class R> struct alignas(8 * sizeof(R)) PairRow {
-    R inv_rho, A_over_rho, C6, qq, A, C, eshift, pad;
+    R inv_rho, A_over_rho, C6, qq, A, C, eshift, lo;
 };
 
 template <int VAR, class R> __device__ __forceinline__ PairRow<R> pair_row(const PairTabT<R> &T, int t)
@@ -681,7 +681,7 @@ template <int VAR, class R> __device__ __forceinline__ PairRow<R> pair_row(const
     PairRow<R> p;
     p.inv_rho = VAR ? T.nl2e_rho[t] : T.inv_rho[t];  // (pair_poly takes the exponent in units of ln 2)
     p.A_over_rho = T.A_over_rho[t]; p.C6 = T.C6[t]; p.qq = T.qq[t];
-    p.A = T.A[t]; p.C = T.C[t]; p.eshift = T.eshift[t]; p.pad = R(0);
+    p.A = T.A[t]; p.C = T.C[t]; p.eshift = T.eshift[t]; p.lo = VAR ? T.nl2e_lo[t] : R(0);
     return p;
 }
 
@@ -753,18 +753,18 @@ __device__ __forceinline__ void pair_poly(const PairTabT<float> &T, const PairRo
     const float r = r2 * rinv;
     const float r4i = r2i * r2i, r8i = r4i * r4i;
     const float u = fmaf(r2, T.r2_us, -1.0f);
-    float p = T.cf[kFitN - 1];
+    float p = T.cf[kFitN<float> - 1];
 #pragma unroll
-    for (int k = kFitN - 2; k >= 0; --k) p = fmaf(p, u, T.cf[k]);
+    for (int k = kFitN<float> - 2; k >= 0; --k) p = fmaf(p, u, T.cf[k]);
     p = fmaf(r2i, rinv, fmaf(-T.fshift, rinv, p));  // one rounding at the size of 1/r^3
     const float a = r * P2.inv_rho;
     float ex = ex2_ftz(a);
     ex = fmaf(ex * 0.69314718f, fmaf(r, P2.inv_rho, -a), ex);
     f_over_r = fmaf(P2.qq, p, fmaf(P2.A_over_rho * ex, rinv, -(P2.C6 * r8i)));
     if (energy) {
-        float q = T.ce[kFitN - 1];
+        float q = T.ce[kFitN<float> - 1];
 #pragma unroll
-        for (int k = kFitN - 2; k >= 0; --k) q = fmaf(q, u, T.ce[k]);
+        for (int k = kFitN<float> - 2; k >= 0; --k) q = fmaf(q, u, T.ce[k]);
         const float ec = (rinv - q) + fmaf(T.fshift, r - T.rc, -T.erfc_rc_over_rc);
         e = fmaf(P2.qq, ec, fmaf(P2.A, ex, fmaf(-P2.C, r4i * r2i, -P2.eshift)));
     } else {
@@ -772,7 +772,52 @@ __device__ __forceinline__ void pair_poly(const PairTabT<float> &T, const PairRo
     }
 }
 
-// FP64 form: library exp / erfc / sqrt (the reference-accuracy path)
+// The same in FP64, variant 1: fits of degree 15 (accurate to 5e-16 of the Coulomb term
+// at the cutoff, else variant 0), 1/r from the FP32 value by one step of third order,
+// e^{-r/rho} as 2^n 2^f with a degree-11 interpolant of 2^f.  The FP64 form is bound by the
+// FP64 pipes (83 % busy on 1728 ions, ~155 of their instructions a list entry with the
+// library's exp, erfc, sqrt and division): this form issues ~60 and takes 76.6 us a step
+// there instead of 159 (64 ions: 20.4 instead of 32).  Its error against 113-bit
+// arithmetic is no larger (MgO and LiH of 64 and 216 ions, 12 seeds: forces 1.03e-14
+// relative L2 instead of 1.05e-14, both from the rounding of the positions; energy
+// 1.0e-16 instead of 1.8e-16): 1/r^2 rounds once from the exact y^2, the fits are made in
+// double-double.
+__device__ __forceinline__ void pair_poly(const PairTabT<double> &T, const PairRow<double> &P2, double r2,
+                                          double &f_over_r, double &e, bool energy)
+{
+    const double y = (double)rsqrt_ftz((float)r2), t = y * y;  // (exact: 24 bits squared)
+    const double d = fma(-r2, t, 1.0);
+    const double rinv = fma(y * d, fma(0.375, d, 0.5), y), r2i = fma(t, fma(d, d, d), t);
+    const double r = r2 * rinv, r4i = r2i * r2i;
+    const double u = fma(r2, T.r2_us, -1.0);
+    double p = T.cf[kFitN<double> - 1];
+#pragma unroll
+    for (int k = kFitN<double> - 2; k >= 0; --k) p = fma(p, u, T.cf[k]);
+    p = fma(r2i, rinv, fma(-T.fshift, rinv, p));
+    // 2^a, a = -r log2(e)/rho: a = n + f, n the nearest integer (the low word of a + 1.5
+    // 2^52), f without the rounding of a
+    const double sh = fma(r, P2.inv_rho, 6755399441055744.0), nd = sh - 6755399441055744.0;
+    const double f = fma(r, P2.lo, fma(r, P2.inv_rho, -nd));
+    const int n = max(__double2loint(sh), -1000);
+    double ex = T.ex2c[kExpN - 1];
+#pragma unroll
+    for (int k = kExpN - 2; k >= 0; --k) ex = fma(ex, f, T.ex2c[k]);
+    ex = __hiloint2double(__double2hiint(ex) + (n << 20), __double2loint(ex));
+    f_over_r = fma(P2.qq, p, fma(P2.A_over_rho * ex, rinv, -(P2.C6 * (r4i * r4i))));
+    if (energy) {
+        double q = T.ce[kFitN<double> - 1];
+#pragma unroll
+        for (int k = kFitN<double> - 2; k >= 0; --k) q = fma(q, u, T.ce[k]);
+        // (ce_lo: what the rounding of ce[0], ce[1] dropped; the charge inside the cutoff is
+        // far from neutral, so a constant of 1e-17 per pair shows in the sum over pairs)
+        const double ec = (rinv - q) + fma(T.fshift, r - T.rc, -fma(T.ce_lo[1], u, T.erfc_rc_over_rc + T.ce_lo[0]));
+        e = fma(P2.qq, ec, fma(P2.A, ex, fma(-P2.C, r4i * r2i, -P2.eshift)));
+    } else {
+        e = 0.0;
+    }
+}
+
+// FP64 form: library exp / erfc / sqrt (any alpha r_cut)
 template <class R>
 __device__ __forceinline__ void pair_eval(const PairTabT<R> &T, const PairRow<R> &P2, R r2, R &f_over_r, R &e,
                                           bool energy = true)
@@ -1092,11 +1137,14 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
             // the raw difference (the box exceeds r_cut/2 + skin)
             const double pd[3] = {(double)pj.x - (double)hp.x, (double)pj.y - (double)hp.y, (double)pj.z - (double)hp.z};
             R dv[3];
+            // (the shift is put together from the edge's words: no FP64 operation)
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const int code = (int)((e >> (26 + 2 * c)) & 3u);
-                const int m = (code == 3) ? -1 : (code == 2) ? (pd[c] > 0.0 ? -2 : 2) : code;
-                dv[c] = (R)(pd[c] + m * RP.box[c]) * lam;
+                const int hi = __double2hiint(RP.box[c]) + (code == 2 ? 1 << 20 : 0), lo = __double2loint(RP.box[c]);
+                const bool neg = code == 3 || (code == 2 && __double2hiint(pd[c]) > 0);
+                const double shift = __hiloint2double(code ? hi | (neg ? (int)0x80000000 : 0) : 0, code ? lo : 0);
+                dv[c] = (R)(pd[c] + shift) * lam;
             }
             g.dx = dv[0]; g.dy = dv[1]; g.dz = dv[2];
             g.tj = (int)pj.w;
@@ -1551,6 +1599,7 @@ static cudaError_t step_prepare_lanes(MdLaunch &m, int stage_entries)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     m.step_smem = (size_t)stage_entries * (m.mixed ? sizeof(int4) : sizeof(D4));
+    if (!m.mixed && m.variant) return step_prepare_variant<PM_BOX64, double, LPA, 1>(m, nsm);
     if (!m.mixed) return step_prepare_variant<PM_BOX64, double, LPA, 0>(m, nsm);
     if (m.variant == 2) return step_prepare_variant<PM_FIX, float, LPA, 2>(m, nsm);
     if (m.variant == 1) return step_prepare_variant<PM_FIX, float, LPA, 1>(m, nsm);
@@ -1603,6 +1652,7 @@ static cudaError_t step_force_lanes(const Dev &d, const MdLaunch &m, const PairT
     if (m.mixed && m.variant == 2) return step_any<PM_FIX, float, LPA, 2>(d, m, Tf, kick, j, cur, adv, rec, st);
     if (m.mixed && m.variant == 1) return step_any<PM_FIX, float, LPA, 1>(d, m, Tf, kick, j, cur, adv, rec, st);
     if (m.mixed) return step_any<PM_FIX, float, LPA, 0>(d, m, Tf, kick, j, cur, adv, rec, st);
+    if (m.variant) return step_any<PM_BOX64, double, LPA, 1>(d, m, Td, kick, j, cur, adv, rec, st);
     return step_any<PM_BOX64, double, LPA, 0>(d, m, Td, kick, j, cur, adv, rec, st);
 }
 

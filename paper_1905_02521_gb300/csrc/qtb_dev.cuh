@@ -26,7 +26,9 @@ constexpr int kFixBits = 30;         // fixed-point positions: box edge = 2^30 u
 constexpr int kMaxTypes = 4;
 constexpr int kExtMaxP = 8;          // external potentials: longest ring carried through many steps a launch
 constexpr int kExtRow = 16;          // doubles of a row of Dev::ext_part
-constexpr int kFitN = 10;            // coefficients of the FP32 Coulomb fits (degree 9)
+// coefficients of the Coulomb fits (degree 9 in FP32, 15 in FP64) and of 2^f (FP64)
+template <class R> constexpr int kFitN = sizeof(R) == 4 ? 10 : 16;
+constexpr int kExpN = 12;
 constexpr int kWarpsPerForceCta = 8;  // warps of the list build kernel
 
 // partial-sum slots
@@ -149,11 +151,12 @@ template <class R> struct PairTabT {
     R alpha2_l2e, erfc_us;
     R rl2;                            // (r_cut + skin)^2: neighbour-list radius
     R erfc_c[12];
-    // FP32 form, variants 1 and 2 of the step kernel: with x = alpha r and u = r^2 r2_us - 1,
+    // polynomial variants of the step kernel (pair_poly): with x = alpha r and u = r^2 r2_us - 1,
     // the Chebyshev fits (monomials in u) of -alpha^3 (erf x - 2 x e^{-x^2}/sqrt(pi))/x^3 (cf)
-    // and alpha erf(x)/x (ce); nl2e_rho = -log2(e)/rho
-    R r2_us, cf[kFitN], ce[kFitN];
-    R nl2e_rho[kMaxTypes * kMaxTypes];
+    // and alpha erf(x)/x (ce); nl2e_rho = -log2(e)/rho; 2^f on |f| <= 1/2 (FP64 form)
+    R r2_us, cf[kFitN<R>], ce[kFitN<R>], ce_lo[2];
+    R nl2e_rho[kMaxTypes * kMaxTypes], nl2e_lo[kMaxTypes * kMaxTypes];  // (lo: its rounding error)
+    R ex2c[kExpN];
     R hdt_m[kMaxTypes];               // dt / (2 m mvv2e)
     R ext_k[kMaxTypes];               // HARMONIC: m mvv2e w0^2
     R ext_V0, ext_ia2;                // DOUBLEWELL: V0, 1/a^2

@@ -68,9 +68,9 @@ struct MdLaunch {
     int nm_big;           // ring-polymer integrator with 32 atoms per CTA (large contexts)
     int lanes;            // lanes per bead-atom of the step kernel of steps that are not recorded (8, 16, 32, 128)
     int step_grid[4];     // resident CTAs of the step kernel, by (adv, rec)
-    int variant;          // step kernel variant of the mixed form: 0 any alpha r_cut (exponential and
-                          // erfc polynomial), 1 the Coulomb term as one polynomial in r^2, 2 the
-                          // same with list displacements by minimum image (fixed cells all larger
+    int variant;          // step kernel variant: 0 any alpha r_cut (exponential and erfc), 1 the
+                          // Coulomb term as one polynomial in r^2, 2 (mixed form) the same with
+                          // list displacements by minimum image (fixed cells all larger
                           // than 2 (r_cut + 2 skin))
     size_t step_smem;     // its dynamic shared memory (list build staging chunk)
 };

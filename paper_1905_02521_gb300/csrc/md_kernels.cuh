@@ -467,39 +467,56 @@ __device__ void sort_phase(const Dev &d, int cur, int *keys)
     }
 }
 
-// List build.  One CTA per home cell: its warps stage the stencil cells
-// (sorted slots; image shift added, fixed point + m 2^30 in wrapping int32
-// arithmetic; the list entry, see kNbIdx, in the last word) chunk by chunk, and for
-// each chunk every warp takes one home bead-atom at a time, scans the flat
-// staged array and appends the entries within r_cut + skin to the bead-atom's
-// list, so that a list is in stencil scan order.
+// List build.  One CTA per home cell, or `parts` CTAs that each take every parts-th
+// group of its bead-atoms while the grid has more CTAs than there are cells: its warps
+// stage the stencil cells (sorted slots; image shift added, fixed point + m 2^30 in
+// wrapping int32 arithmetic; the list entry, see kNbIdx, in the last word) chunk by
+// chunk, and for each chunk every warp takes one home bead-atom at a time, scans the flat
+// staged array and appends the entries within r_cut + skin to the bead-atom's list, so
+// that a list is in stencil scan order.  Bound by its instructions on many bead-atoms
+// (~1700 candidates each) and by the chain of one warp's scans on few; a rebuild, with
+// its three grid barriers, measured before (one CTA a cell, one scan for each half of the
+// list) and now: 64 ions 28.9 -> 22.3 us, 8000 46.4 -> 38.9, 32768 132 -> 114, 1728 at
+// constant pressure 74 -> 61, LiH 13824 bead-atoms 73 -> 60, 55296 213 -> 170; FP64 form
+// 64 ions 82 -> 38, 1728 162 -> 100.
 constexpr int kStencilHalf = 2;
 constexpr int kStencil = (2 * kStencilHalf + 1) * (2 * kStencilHalf + 1) * (2 * kStencilHalf + 1);
+
+constexpr int kMaxParts = 8;
+
+// where a row keeps its k-th entry: blocks in the order of the step kernel's loads, see kCols
+__device__ __forceinline__ int list_at(int k)
+{
+    return (k & ~(kColBlock - 1)) + (k & (kCols - 1)) * kColNE + (k / kCols) % kColNE;
+}
 
 // shared memory of build_cell (besides the staging chunk)
 struct BuildSmem {
     int soff[kStencil + 1], scell[kStencil], sbase[kStencil], simg[kStencil][3];
-    int scount[kMaxCellCap];
+    unsigned scount[kMaxCellCap];  // entries within r_cut + 2^16 parked ones (both < kMaxCellCap kStencil)
 };
 
 template <int PM, class R>
-__device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, int cur, void *stage_mem, BuildSmem &B)
+__device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, int part, int parts, int cur, void *stage_mem,
+                           BuildSmem &B)
 {
     typedef typename std::conditional<PM == PM_FIX, int4, D4>::type E4;
     constexpr int SH = kStencilHalf, SW = 2 * kStencilHalf + 1;
-    int *soff = B.soff, *scell = B.scell, *scount = B.scount;
+    int *soff = B.soff, *scell = B.scell;
+    unsigned *scount = B.scount;
     int (*simg)[3] = B.simg;
     E4 *stage = reinterpret_cast<E4 *>(stage_mem);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
     __syncthreads();  // the previous cell of this CTA is done with the shared memory
     const int cnt = d.ccount[cell];
-    if (cnt == 0) return;  // uniform over the CTA
+    if (part * nwarp >= max(cnt, 1)) return;  // uniform over the CTA
     const DRep RP = d.rep[d.cell_rep[cell]];
     const int lc = cell - RP.cell0;
-    if (threadIdx.x == 0) d.cnt[cell] = 0;  // for the next rebuild's binning (the scan has read it)
+    if (threadIdx.x == 0 && part == 0) d.cnt[cell] = 0;  // for the next rebuild's binning (the scan has read it)
+    if (cnt == 0) return;
     // the cell's bead-atoms: their slots, and the packed positions there (the other
     // buffer gets the types: the one-bead step writes only coordinates to it)
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+    for (int t = part * (int)blockDim.x + threadIdx.x; t < cnt; t += parts * blockDim.x) {
         const size_t o = (size_t)cell * d.cap + t;
         const int sl = d.cbase[cell] + t;
         E4 p = reinterpret_cast<const E4 *>(d.cpos)[o];
@@ -549,19 +566,23 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, int cur, void *
     // entries (a multiple of 64); each home slot's list grows chunk by chunk
     const int total = soff[kStencil];
     const int CH = d.stage_cap;
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) scount[t] = 0;
+    for (int t = threadIdx.x; t < cnt; t += blockDim.x) scount[t] = 0u;
     // physical distances (isothermal-isobaric: the reference cell scaled by lam)
     const R lam = (d.npt && d.npt[RP.sys].on) ? (R)d.npt[RP.sys].lam : R(1);
     const R sx = (R)RP.fix_scale[0] * lam, sy = (R)RP.fix_scale[1] * lam, sz = (R)RP.fix_scale[2] * lam;
     const unsigned lt = (1u << lane) - 1u;
     const int maxnb = d.maxnb;
-    // pass 0 lists the entries within r_cut, pass 1 those of the skin shell, so
-    // that the shell entries close every list (the force loop can skip them)
-    for (int pass = 0; pass < 2; ++pass)
+    // The entries within r_cut open a list and those of the skin shell close it, so that
+    // the force loop can skip them.  One scan finds both: it parks the shell entries at the
+    // end of the row, backwards, and they move up when the first part's length is known.
+    // A second scan lists them only if a row of this CTA was too full for that.
+    bool rescan = false;
+    for (int pass = 0; pass < (rescan ? 2 : 1); ++pass) {
     for (int c0 = 0; c0 < total; c0 += CH) {
         const int cn = min(CH, total - c0);
         const int padded = (cn + 63) & ~63;
         __syncthreads();  // the previous chunk is scanned
+        if (pass == 0 || total > CH) {  // (one chunk: still staged)
         // flat staging: every thread first issues all of its (independent) loads,
         // then shifts by the image and stores
         constexpr int U = 4;
@@ -615,12 +636,13 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, int cur, void *
             else reinterpret_cast<D4 *>(stage)[e] = D4{-1e30, -1e30, -1e30, 0.0};
         }
         __syncthreads();
-        for (int slot = warp; slot < cnt; slot += nwarp) {
+        }
+        for (int slot = part * nwarp + warp; slot < cnt; slot += parts * nwarp) {
             // the home bead-atom: its own cell, image 0
             const E4 hp = reinterpret_cast<const E4 *>(d.cpos)[(size_t)cell * d.cap + slot];
             const int gi = d.cidx[(size_t)cell * d.cap + slot];
             unsigned *row = d.nbr + (size_t)gi * maxnb;
-            int n = scount[slot];
+            int n = scount[slot] & 0xffffu, m = scount[slot] >> 16;
             auto test = [&](const E4 &pj) {
                 R dx, dy, dz;
                 if (PM == PM_FIX) {
@@ -635,27 +657,66 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, int cur, void *
                 const R r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                 // the home bead-atom itself (r2 == 0) and the sentinels fail
                 const bool take = pass == 0 ? (r2 < rc2 && r2 > R(0)) : (r2 >= rc2 && r2 < rl2);
-                const unsigned m = __ballot_sync(0xffffffffu, take);
+                const unsigned bt = __ballot_sync(0xffffffffu, take);
                 if (take) {
-                    const int k = n + __popc(m & lt);
-                    // (blocks in the order of the step kernel's loads, see kCols)
-                    if (k < maxnb) row[(k & ~(kColBlock - 1)) + (k & (kCols - 1)) * kColNE + (k / kCols) % kColNE] = (unsigned)pj.w;
+                    const int k = n + __popc(bt & lt);
+                    if (k < maxnb) row[list_at(k)] = (unsigned)pj.w;
                 }
-                n += __popc(m);
+                n += __popc(bt);
+                if (pass) return;
+                const bool shell = r2 >= rc2 && r2 < rl2;
+                const unsigned bs = __ballot_sync(0xffffffffu, shell);
+                if (shell) {  // never onto the first part's blocks
+                    const int at = maxnb - 1 - (m + __popc(bs & lt));
+                    if (at >= ((n + kColBlock - 1) & ~(kColBlock - 1))) row[at] = (unsigned)pj.w;
+                }
+                m += __popc(bs);
             };
             for (int e0 = 0; e0 < padded; e0 += 64) {
                 const E4 pa = stage[e0 + lane], pb = stage[e0 + 32 + lane];
                 test(pa);
                 test(pb);
             }
-            if (lane == 0) scount[slot] = n;
+            __syncwarp();
+            if (lane == 0) scount[slot] = (unsigned)n | ((unsigned)m << 16);
         }
+    }
+    if (pass) break;
+    __syncwarp();
+    // the parked entries, kMove rounds of 32 at a time
+    constexpr int kMove = 4;
+    bool full = false;
+    for (int slot = part * nwarp + warp; slot < cnt; slot += parts * nwarp) {
+        const int n = scount[slot] & 0xffffu, m = scount[slot] >> 16;
+        // the parked ones are intact, and no batch's targets reach a later batch's sources
+        const int end = m > 32 * kMove ? n + m : n;
+        if (((end + kColBlock - 1) & ~(kColBlock - 1)) > maxnb - m) full = true;
+    }
+    rescan = __syncthreads_or(full);
+    if (rescan) continue;
+    for (int slot = part * nwarp + warp; slot < cnt; slot += parts * nwarp) {
+        const int n = scount[slot] & 0xffffu, m = scount[slot] >> 16;
+        unsigned *row = d.nbr + (size_t)d.cidx[(size_t)cell * d.cap + slot] * maxnb;
+        for (int b = 0; b < m; b += 32 * kMove) {
+            unsigned w[kMove];
+#pragma unroll
+            for (int q = 0; q < kMove; ++q) w[q] = b + 32 * q + lane < m ? row[maxnb - 1 - (b + 32 * q + lane)] : 0u;
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < kMove; ++q)
+                if (b + 32 * q + lane < m) row[list_at(n + b + 32 * q + lane)] = w[q];
+        }
+        __syncwarp();
+        if (lane == 0) scount[slot] = (unsigned)(n + m);
+    }
     }
     __syncthreads();
     for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+        if (t / nwarp % parts != part) continue;
         const int gi = d.cidx[(size_t)cell * d.cap + t];
-        d.nnb[gi] = min(scount[t], maxnb);
-        if (scount[t] > maxnb) atomicOr(d.err, (unsigned)ERR_NBR_OVERFLOW);
+        const int n = scount[t] & 0xffffu;  // (a second scan leaves the parked count above it)
+        d.nnb[gi] = min(n, maxnb);
+        if (n > maxnb) atomicOr(d.err, (unsigned)ERR_NBR_OVERFLOW);
     }
 }
 
@@ -1534,11 +1595,21 @@ __global__ void __launch_bounds__(32 * kListWarps, sizeof(R) == 4 ? (REC ? 4 : L
         scan_phase(d, cur, B.soff);
         sort_phase<PM>(d, cur, reinterpret_cast<int *>(fsm));
         grid_barrier(d);
-        for (int s = 0; s < d.nsys; ++s) {  // the cells of the requesting systems
-            if (!d.rebuild_all && d.rflag[cur * d.nsys + s] == 0u) continue;  // uniform over the grid
-            const int c0 = d.sys[s].cell0, c1 = d.sys[s].cell1, nb = (int)gridDim.x;
-            for (int cell = c0 + (((int)blockIdx.x - c0) % nb + nb) % nb; cell < c1; cell += nb)
-                build_cell<PM, R>(d, T.rc2, sizeof(R) == 4 ? (R)d.sys[s].rl2_f : (R)d.sys[s].rl2, cell, cur, fsm, B);
+        // the cells of the requesting systems, dealt over the CTAs; a cell is shared by
+        // several while the grid has more CTAs than there are cells
+        const int nb = (int)gridDim.x;
+        int cells = 0;
+        for (int s = 0; s < d.nsys; ++s)  // (all conditions uniform over the grid)
+            if (d.rebuild_all || d.rflag[cur * d.nsys + s] != 0u) cells += d.sys[s].cell1 - d.sys[s].cell0;
+        const int parts = max(1, min(kMaxParts, nb / max(cells, 1)));
+        int at = (int)blockIdx.x;  // this CTA's next item, counted from the system's first
+        for (int s = 0; s < d.nsys; ++s) {
+            if (!d.rebuild_all && d.rflag[cur * d.nsys + s] == 0u) continue;
+            const int c0 = d.sys[s].cell0, items = (d.sys[s].cell1 - c0) * parts;
+            for (; at < items; at += nb)
+                build_cell<PM, R>(d, T.rc2, sizeof(R) == 4 ? (R)d.sys[s].rl2_f : (R)d.sys[s].rl2, c0 + at / parts,
+                                  at % parts, parts, cur, fsm, B);
+            at -= items;
         }
         grid_barrier(d);
         // the per-system requests were read by every phase: consumed now (their

@@ -476,9 +476,9 @@ __device__ void sort_phase(const Dev &d, int cur, int *keys)
 // that a list is in stencil scan order.  Bound by its instructions on many bead-atoms
 // (~1700 candidates each) and by the chain of one warp's scans on few; a rebuild, with
 // its three grid barriers, measured before (one CTA a cell, one scan for each half of the
-// list) and now: 64 ions 28.9 -> 22.3 us, 8000 46.4 -> 38.9, 32768 132 -> 114, 1728 at
-// constant pressure 74 -> 61, LiH 13824 bead-atoms 73 -> 60, 55296 213 -> 170; FP64 form
-// 64 ions 82 -> 38, 1728 162 -> 100.
+// list) and now: 64 ions 28.9 -> 21.3 us, 8000 46.4 -> 38.2, 32768 132 -> 112, 1728 at
+// constant pressure 74 -> 57, LiH 13824 bead-atoms 73 -> 58, 55296 213 -> 165; FP64 form
+// 64 ions 82 -> 37, 1728 162 -> 94.
 constexpr int kStencilHalf = 2;
 constexpr int kStencil = (2 * kStencilHalf + 1) * (2 * kStencilHalf + 1) * (2 * kStencilHalf + 1);
 
@@ -656,6 +656,7 @@ __device__ void build_cell(const Dev &d, R rc2, R rl2, int cell, int part, int p
                 }
                 const R r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                 // the home bead-atom itself (r2 == 0) and the sentinels fail
+                if (!__any_sync(0xffffffffu, r2 < rl2)) return;  // (55296 bead-atoms: 165 us a rebuild, 170 without)
                 const bool take = pass == 0 ? (r2 < rc2 && r2 > R(0)) : (r2 >= rc2 && r2 < rl2);
                 const unsigned bt = __ballot_sync(0xffffffffu, take);
                 if (take) {

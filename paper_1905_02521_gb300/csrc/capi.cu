@@ -739,8 +739,10 @@ int setup_fourier(qtb_ctx *c, const std::vector<DSpec> &spec)
 }
 
 // The FP64 filter of a system switches to the fast convolution at this half
-// length, as long as its spectra stay within the limit.
-constexpr int kFftMinK = 64;
+// length, as long as its spectra stay within the limit.  Measured, 32769 dofs, ms per
+// 256 steps (steps included), direct / fast: K = 16 1.83 / 2.35, 32 2.30 / 2.35,
+// 64 3.23 / 2.35, 128 5.11 / 2.36, 1024 31.3 / 2.71.
+constexpr int kFftMinK = 40;
 constexpr size_t kFftMaxRing = (size_t)16 << 30;
 
 // (re)build taps of every system from hs[].mode/n_taps/omega_max
@@ -896,9 +898,9 @@ double effective_skin(const qtb_params *p, double T)
 // 8000: 15.1 / 10.7 / 14.7, 10648: 14.4 / 16.9 / 17.9, 32768: 36.9 / 32.0, 64000: 62.4 /
 // 62.8; ring polymers (7 CTAs per SM) 1728: 10.8 / 9.7 / 9.3, 4096: 13.9 / 13.4 / 14.9,
 // 55296: 76.4 / 70.7, 221184: 231 / 236, 864000: 887 / 917; FP64 form (bound by the
-// FP64 pipes, so its work is spread over the SMs) 64: 103 / 58 / 38 / 20, 512: 92 / 51 /
-// 39 / 29, 1728: 123 / 103 / 89 / 77, 2744: 200 / 163 / 175 / 123, 4096: 278 / 164 / 176 /
-// 172, 8000: 326 / 324 / 347 / 324.
+// FP64 pipes, so its work is spread over the SMs) 64: 97 / 51 / 32 / 14, 512: 92 / 51 /
+// 39 / 30, 1728: 124 / 103 / 90 / 76, 2744: 200 / 163 / 175 / 123, 4096: 298 / 164 / 176 /
+// 164, 8000: 327 / 324 / 347 / 324.
 int default_lanes(long long n, bool fp64, bool one_bead, int nsm)
 {
     if (fp64) return n <= 24LL * nsm ? 128 : 16;

@@ -839,7 +839,7 @@ __device__ __forceinline__ void pair_poly(const PairTabT<float> &T, const PairRo
 // e^{-r/rho} as 2^n 2^f with a degree-11 interpolant of 2^f.  The FP64 form is bound by the
 // FP64 pipes (83 % busy on 1728 ions, ~155 of their instructions a list entry with the
 // library's exp, erfc, sqrt and division): this form issues ~60 and takes 76.6 us a step
-// there instead of 159 (64 ions: 20.4 instead of 32).  Its error against 113-bit
+// there instead of 159 (64 ions: 13.5 instead of 32).  Its error against 113-bit
 // arithmetic is no larger (MgO and LiH of 64 and 216 ions, 12 seeds: forces 1.03e-14
 // relative L2 instead of 1.05e-14, both from the rounding of the positions; energy
 // 1.0e-16 instead of 1.8e-16): 1/r^2 rounds once from the exact y^2, the fits are made in

@@ -805,7 +805,9 @@ void launch_white(const Dev &d, int filter_kind, int max_dofp, int nsys, long lo
 }
 
 // the tiled FP32 filter from this half length on (below, the window loads dominate
-// either form), up to what its 8 windows need of shared memory
+// either form), up to what its 8 windows need of shared memory.  Measured, 32769 dofs, ms
+// per 256 steps (steps included), one dof a CTA / tiled: K = 8 0.36 / 0.31, 32 0.40 / 0.33,
+// 128 0.61 / 0.40, 1024 2.71 / 1.09.
 constexpr int kTileMinK = 8;
 constexpr size_t kTileMaxSmem = 220 * 1024;
 

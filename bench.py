@@ -484,7 +484,7 @@ def fp64_form_leg(qtb, torch, systems, params, setup, states, units, n_blocks, c
         qtb.qtb_destroy(ctx)
     t = float(np.sum(ms))
     return {"value": units * BLOCK * n_blocks / (t / 1e3), "unit": UNIT, "ms_per_step": t / n_blocks,
-            "steps": n_blocks, "dtype": "f64", "filter": "fp64 (direct convolution)",
+            "steps": n_blocks, "dtype": "f64", "filter": "fp64 (partitioned convolution)",
             "start": "the mixed form's steady state, lists rebuilt, one warm-up block"}
 
 

@@ -113,6 +113,7 @@ struct qtb_ctx {
     // profiling (events recorded inside the captured block)
     bool profiling = false, capturing = false;
     std::vector<cudaEvent_t> ev;        // pairs: start, stop
+    cudaEvent_t ev_up = nullptr;        // an upload's copies are done
     std::vector<int> ev_cls;            // class of each pair
     size_t ev_used = 0, ev_pairs = 0;
     bool prof_launched = false;
@@ -159,6 +160,7 @@ struct qtb_ctx {
             else cudaFree(ptr);
         }
         for (cudaEvent_t e : ev) cudaEventDestroy(e);
+        if (ev_up) cudaEventDestroy(ev_up);
         if (own_stream) cudaStreamDestroy(st);
     }
 };
@@ -350,8 +352,8 @@ static int decode_err_word(qtb_ctx *c, unsigned e)
 int upload_state(qtb_ctx *c, int s, const double *pos, const double *vel)
 {
     // one copy per array into a staging buffer, the conversion on the device
-    // (k_load_state), one synchronisation: the caller's arrays are borrowed
-    // for the call only (pinned host memory makes the copies plain DMA)
+    // (k_load_state): the caller's arrays are borrowed for the call only (pinned host
+    // memory makes the copies plain DMA), so the call waits for the copies
     if (!pos && !vel) return QTB_OK;
     const HSys &h = c->hs[s];
     const size_t n3 = 3 * (size_t)h.N * h.P;
@@ -363,29 +365,39 @@ int upload_state(qtb_ctx *c, int s, const double *pos, const double *vel)
     double *dp = pos ? c->d_stage : nullptr, *dv = vel ? c->d_stage + n3 : nullptr;
     if (pos) CUDA_TRY(cudaMemcpyAsync(dp, pos, sizeof(double) * n3, cudaMemcpyHostToDevice, c->st));
     if (vel) CUDA_TRY(cudaMemcpyAsync(dv, vel, sizeof(double) * n3, cudaMemcpyHostToDevice, c->st));
+    if (!c->ev_up) CUDA_TRY(cudaEventCreateWithFlags(&c->ev_up, cudaEventDisableTiming));
+    CUDA_TRY(cudaEventRecord(c->ev_up, c->st));
     // once the lists exist, an uploaded position is stored as its periodic copy
     // nearest the reference of the last rebuild (positions are not wrapped between
     // rebuilds): an unchanged state then keeps its lists
     launch_load_state(c->d, c->ml, s, (long long)n3, dp, dv, (c->pair && c->lists_built) ? 1 : 0, c->st);
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaStreamSynchronize(c->st));
+    CUDA_TRY(cudaEventSynchronize(c->ev_up));
     return QTB_OK;
 }
 
-// which: 0 positions, 1 velocities, 2 forces
-int download(qtb_ctx *c, int s, int which, double *out)
+// arrays (0 positions, 1 velocities, 2 forces) of system s, null destinations left out:
+// converted on the device into the staging buffer, then the error word, then (unless it
+// holds an error) the arrays; the conversions are queued behind the work they wait for, so
+// that only copies follow it
+int download(qtb_ctx *c, int s, int n, const int *which, double *const *out)
 {
-    // converted on the device into the staging buffer, one copy, one synchronisation
     const HSys &h = c->hs[s];
     const size_t n3 = 3 * (size_t)h.N * h.P;
-    if (c->stage_n < n3) {
+    if (c->stage_n < 2 * n3) {
         c->d_stage = (double *)c->alloc(sizeof(double) * 2 * n3);  // freed with the context
-        if (!c->d_stage) return fail(QTB_ERR_OOM, "device allocation failed");
+        if (!c->d_stage) {
+            c->stage_n = 0;
+            return fail(QTB_ERR_OOM, "device allocation failed");
+        }
         c->stage_n = 2 * n3;
     }
-    launch_store_state(c->d, c->ml, s, (long long)n3, which, c->d_stage, c->st);
+    for (int k = 0; k < n; ++k)
+        if (out[k]) launch_store_state(c->d, c->ml, s, (long long)n3, which[k], c->d_stage + k * n3, c->st);
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpyAsync(out, c->d_stage, sizeof(double) * n3, cudaMemcpyDeviceToHost, c->st));
+    if (int rc = check_err_word(c)) return rc;
+    for (int k = 0; k < n; ++k)
+        if (out[k]) CUDA_TRY(cudaMemcpyAsync(out[k], c->d_stage + k * n3, sizeof(double) * n3, cudaMemcpyDeviceToHost, c->st));
     CUDA_TRY(cudaStreamSynchronize(c->st));
     return QTB_OK;
 }
@@ -421,7 +433,8 @@ int refresh_forces(qtb_ctx *c)
             launch_refresh_check(c->d, c->ml, cur, c->st);
         }
     }
-    launch_spring(c->d, c->ml, c->st);  // the record's spring term (no integrator ran)
+    // the record's spring term (no integrator ran); one-bead crystals have none
+    if (!c->pair || c->ml.n_ccta) launch_spring(c->d, c->ml, c->st);
     CUDA_TRY(launch_force(c->d, c->ml, c->tabf, c->tab, 0, j, cur, 0, 1, c->st));
     if (!c->pair) launch_reduce(c->d, c->ml, j, -1, c->st);  // the list force kernel reduces itself
     launch_centroid(c->d, c->ml, j, -1, 0, c->st);
@@ -1650,11 +1663,9 @@ int qtb_get_state(qtb_ctx *c, int sys, double *pos, double *vel)
     if (!c) return fail(QTB_ERR_ARG, "null context");
     if (sys < 0 || sys >= (int)c->hs.size()) return fail(QTB_ERR_ARG, "system %d out of range", sys);
     if (int rc0 = ensure_fresh(c)) return rc0;
-    int rc = check_err_word(c);
-    if (rc) return rc;
-    if (pos && (rc = download(c, sys, 0, pos))) return rc;
-    if (vel && (rc = download(c, sys, 1, vel))) return rc;
-    return QTB_OK;
+    const int which[2] = {0, 1};
+    double *const out[2] = {pos, vel};
+    return download(c, sys, 2, which, out);
 }
 
 int qtb_set_state(qtb_ctx *c, int sys, const double *pos, const double *vel)
@@ -1672,9 +1683,8 @@ int qtb_get_forces(qtb_ctx *c, int sys, double *f)
     if (!c || !f) return fail(QTB_ERR_ARG, "null argument");
     if (sys < 0 || sys >= (int)c->hs.size()) return fail(QTB_ERR_ARG, "system %d out of range", sys);
     if (int rc0 = ensure_fresh(c)) return rc0;
-    int rc = check_err_word(c);
-    if (rc) return rc;
-    return download(c, sys, 2, f);
+    const int which = 2;
+    return download(c, sys, 1, &which, &f);
 }
 
 int qtb_get_taps(qtb_ctx *c, int sys, double *h, int max, int *n_out)

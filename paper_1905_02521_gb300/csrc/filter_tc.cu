@@ -255,7 +255,7 @@ __global__ void k_build_toeplitz(Dev d, __nv_bfloat16 *Bt, int Ktot, int Ke)
 
 cudaError_t filter_tc_prepare()
 {
-    return cudaFuncSetAttribute(k_filter_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_BYTES);
+    return allow_dynamic_smem(k_filter_tc, tc::SMEM_BYTES);
 }
 
 void launch_build_toeplitz(const Dev &d, void *Bt, int Ktot, int Ke, cudaStream_t st)

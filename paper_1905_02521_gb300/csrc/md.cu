@@ -550,8 +550,8 @@ static void nm_launch(const Dev &d, const MdLaunch &m, int j, int cur, cudaStrea
 template <int P, int PM, class R>
 static cudaError_t nm_prepare_one(int big)
 {
-    if (big) return cudaFuncSetAttribute(k_integrate_nm<P, PM, R, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nm_smem<P, PM, R>(1));
-    return cudaFuncSetAttribute(k_integrate_nm<P, PM, R, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nm_smem<P, PM, R>(0));
+    if (big) return allow_dynamic_smem(k_integrate_nm<P, PM, R, 1>, nm_smem<P, PM, R>(1));
+    return allow_dynamic_smem(k_integrate_nm<P, PM, R, 0>, nm_smem<P, PM, R>(0));
 }
 
 template <int PM, class R>

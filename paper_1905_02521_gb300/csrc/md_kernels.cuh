@@ -1639,7 +1639,7 @@ __global__ void __launch_bounds__(32 * kListWarps, sizeof(R) == 4 ? (REC ? 4 : L
 template <int PM, class R, int ADV, int REC, int LPA, int VAR>
 static cudaError_t step_prepare_one(size_t smem, int nsm, int &grid)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_step<PM, R, ADV, REC, LPA, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(k_step<PM, R, ADV, REC, LPA, VAR>, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<PM, R, ADV, REC, LPA, VAR>, 32 * kListWarps, smem);

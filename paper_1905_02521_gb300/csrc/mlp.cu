@@ -401,7 +401,7 @@ int qtb_kappa_model_grad(qtb_kappa_model *M, const float *x, const float *t, int
     cudaMemset(st, 0, sizeof(AdamState));
     cudaMemcpy(dx, x, sizeof(float) * 2 * n, cudaMemcpyHostToDevice);
     cudaMemcpy(dt, t, sizeof(float) * n, cudaMemcpyHostToDevice);
-    cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_grad_smem());
+    allow_dynamic_smem(k_mlp_grad, mlp_grad_smem());
     k_mlp_grad<<<nblk, kGradThreads, mlp_grad_smem()>>>(M->w, reinterpret_cast<const float2 *>(dx), dt, n,
                                                         1.0f / n, gp, lp);
     k_mlp_reduce_adam<<<(kNP + 31) / 32, 256>>>(gp, nblk, M->w, M->m, M->v, gd, lp, ld, st, 0, 0.f, 1.f, 1, 0);
@@ -462,7 +462,7 @@ int qtb_kappa_model_train(qtb_kappa_model *M, const int *P_list, int nP, int n_p
     cudaMemcpy(dx, X.data(), sizeof(float) * X.size(), cudaMemcpyHostToDevice);
     cudaMemcpy(dt, Tg.data(), sizeof(float) * Tg.size(), cudaMemcpyHostToDevice);
     cudaMemcpy(dxv, Xv.data(), sizeof(float) * Xv.size(), cudaMemcpyHostToDevice);
-    cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_grad_smem());
+    allow_dynamic_smem(k_mlp_grad, mlp_grad_smem());
     cudaStream_t sm;
     cudaStreamCreateWithFlags(&sm, cudaStreamNonBlocking);
     cudaEvent_t e0, e1;

@@ -828,14 +828,11 @@ void launch_filter_simt(const Dev &d, int filter_kind, int max_dofp, int nsys, i
 
 cudaError_t filter_simt_prepare(int Kmax)
 {
-    size_t sm = sizeof(double) * (kBlockSteps + 3 * Kmax + 1);
-    cudaError_t e = cudaFuncSetAttribute(k_filter_simt<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_filter_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::min(tile_smem(Kmax), kTileMaxSmem));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_filter_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(sm / 2 + 16));
+    const size_t taps = kBlockSteps + 3 * (size_t)Kmax + 1;
+    cudaError_t e = allow_dynamic_smem(k_filter_simt<double>, sizeof(double) * taps);
+    if (e == cudaSuccess) e = allow_dynamic_smem(k_filter_tile, std::min(tile_smem(Kmax), kTileMaxSmem));
+    if (e == cudaSuccess) e = allow_dynamic_smem(k_filter_simt<float>, sizeof(float) * taps);
+    return e;
 }
 
 void launch_spectrum_taps(const DSpec *spec, int nsys, int Kmax, double *S, double *cs, double *h64, float *h32,
@@ -880,11 +877,8 @@ size_t fourier_smem(int n, int fp64) { return (size_t)2 * kSegPairs * 2 * n * (f
 
 cudaError_t fourier_prepare(int n)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_fourier<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)fourier_smem(n, 0));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_fourier<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)fourier_smem(n, 1));
+    const cudaError_t e = allow_dynamic_smem(k_fourier<float, float>, fourier_smem(n, 0));
+    return e != cudaSuccess ? e : allow_dynamic_smem(k_fourier<double, double>, fourier_smem(n, 1));
 }
 
 void launch_spectrum_seg(const DSpec *spec, int nsys, int n, void *sq, int fp64, cudaStream_t st)

@@ -227,7 +227,7 @@ size_t fft_table_values(int nslots, int nsys) { return 2 * (size_t)kFftN * ((siz
 
 cudaError_t filter_fft_prepare()
 {
-    return cudaFuncSetAttribute(k_filter_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFftSmem);
+    return allow_dynamic_smem(k_filter_fft, kFftSmem);
 }
 
 void launch_fft_tables(const Dev &d, const double *taps64, void *tw, void *G, cudaStream_t st)

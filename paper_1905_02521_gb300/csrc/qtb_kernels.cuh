@@ -16,6 +16,24 @@ struct DSpec {
     double ymax, y0;
 };
 
+// Lets a kernel be launched with `need` bytes of dynamic shared memory.  The limit belongs
+// to the function on the device, so to every context of the process: it is set to the most
+// the device allows beside the kernel's static part, never to what one context needs (the
+// next one's smaller need would then turn down the first one's launches).
+template <class F> cudaError_t allow_dynamic_smem(F kernel, size_t need)
+{
+    int dev = 0, optin = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    const int most = optin - (int)a.sharedSizeBytes;
+    if ((long long)need > most) return cudaErrorInvalidValue;
+    if (a.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // capi.cu: record the message returned by qtb_last_error(); returns code
 int set_last_error(int code, const char *msg);
 

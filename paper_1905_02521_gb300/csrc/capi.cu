@@ -40,7 +40,10 @@ int fail(int code, const char *fmt, ...)
 #define CUDA_TRY(expr)                                                                      \
     do {                                                                                    \
         cudaError_t e_ = (expr);                                                            \
-        if (e_ != cudaSuccess) return fail(QTB_ERR_CUDA, "%s: %s", #expr, cudaGetErrorString(e_)); \
+        if (e_ != cudaSuccess) {                                                            \
+            (void)cudaGetLastError(); /* reported here: not the next call's */              \
+            return fail(QTB_ERR_CUDA, "%s: %s", #expr, cudaGetErrorString(e_));             \
+        }                                                                                   \
     } while (0)
 
 long long roundup(long long a, long long b) { return (a + b - 1) / b * b; }
@@ -404,19 +407,31 @@ int download(qtb_ctx *c, int s, int n, const int *which, double *const *out)
 
 // ---- pipeline pieces -------------------------------------------------------
 
-void set_clock(qtb_ctx *c, long long b)
+int set_clock(qtb_ctx *c, long long b)
 {
     if (c->dclock != b) {
         launch_setclock(c->d, b, c->st);
+        CUDA_TRY(cudaGetLastError());
         c->dclock = b;
     }
+    return QTB_OK;
+}
+
+// after a failed call: what the host noted of the device's clock, the noise ring and the
+// coloured noise may not have happened, so all of it is made again (the noise is a function
+// of the block index) before it is used
+void forget_noise(qtb_ctx *c)
+{
+    c->dclock = -1;
+    c->ring_hi = c->ring_lo = c->eta_blk = c->eta_seg = LLONG_MIN;
+    c->graph_dirty = true;
 }
 
 // forces (and energies) at the current positions, the lists rebuilt where needed
 // (all of them at the first evaluation); no velocity kick
 int refresh_forces(qtb_ctx *c)
 {
-    set_clock(c, floor_div(c->step, kBlockSteps));
+    if (int rc = set_clock(c, floor_div(c->step, kBlockSteps))) return rc;
     const int j = (int)(c->step - c->dclock * kBlockSteps) - 1;
     const int cur = (int)(c->step & 1);  // positions of step s live in pos[s & 1]
     if (c->pair) {
@@ -442,13 +457,15 @@ int refresh_forces(qtb_ctx *c)
     return QTB_OK;
 }
 
-void gen_white(qtb_ctx *c, long long blk)
+int gen_white(qtb_ctx *c, long long blk)
 {
     if (c->fft) launch_white_fft(c->d, c->max_dofp, blk, c->st);
     if (c->direct) launch_white(c->d, c->fk, c->max_dofp, c->d.nsys, blk, c->st);
+    CUDA_TRY(cudaGetLastError());
+    return QTB_OK;
 }
 
-void filter_block(qtb_ctx *c)
+int filter_block(qtb_ctx *c)
 {
     if (c->fk == FK_BF16)
         launch_filter_tc(c->d, &c->tmA, &c->tmB, c->n_tiles, c->d_tiles, c->st);
@@ -456,6 +473,8 @@ void filter_block(qtb_ctx *c)
         launch_filter_fft(c->d, c->max_dofp, c->st);
     if (c->fk != FK_BF16 && c->direct)
         launch_filter_simt(c->d, c->fk, c->max_dofp, c->d.nsys, c->Kmax, c->st);
+    CUDA_TRY(cudaGetLastError());
+    return QTB_OK;
 }
 
 // cuTensorMapEncodeTiled from the driver library, resolved at run time so that
@@ -524,36 +543,40 @@ int setup_tc(qtb_ctx *c)
 }
 
 // make the ring hold white blocks lo .. hi (hi - lo < nslots)
-void ensure_ring(qtb_ctx *c, long long lo, long long hi)
+int ensure_ring(qtb_ctx *c, long long lo, long long hi)
 {
     long long from = lo;
     const bool have = (c->ring_hi != LLONG_MIN && c->ring_lo <= lo && c->ring_hi >= lo - 1);
     if (have) from = c->ring_hi + 1;
-    for (long long blk = from; blk <= hi; ++blk) gen_white(c, blk);
+    for (long long blk = from; blk <= hi; ++blk)
+        if (int rc = gen_white(c, blk)) return rc;
     if (!have) c->ring_lo = lo;
     if (!have || hi > c->ring_hi) c->ring_hi = std::max(hi, have ? c->ring_hi : hi);
     c->ring_lo = std::max(c->ring_lo, c->ring_hi - c->d.nslots + 1);
+    return QTB_OK;
 }
 
 // make eta hold block b (ring then holds blocks b-Kb .. b+Kb)
-void ensure_eta(qtb_ctx *c, long long b)
+int ensure_eta(qtb_ctx *c, long long b)
 {
     if (c->gen == QTB_GEN_FOURIER) {
         const long long seg = floor_div(b, c->seg_blocks);
-        set_clock(c, b);
+        if (int rc = set_clock(c, b)) return rc;
         if (c->eta_seg != seg) {
             launch_fourier(c->d, c->mixed ? 0 : 1, c->max_dofp, c->d.nsys, c->d_sq, c->d_tw,
                            kBlockSteps * c->seg_blocks, 1, c->st);
+            CUDA_TRY(cudaGetLastError());
             c->eta_seg = seg;
         }
         c->eta_blk = b;
-        return;
+        return QTB_OK;
     }
-    if (c->eta_blk == b) return;
-    ensure_ring(c, b - c->d.Kb, b + c->d.Kb);
-    set_clock(c, b);
-    filter_block(c);
+    if (c->eta_blk == b) return QTB_OK;
+    if (int rc = ensure_ring(c, b - c->d.Kb, b + c->d.Kb)) return rc;
+    if (int rc = set_clock(c, b)) return rc;
+    if (int rc = filter_block(c)) return rc;
     c->eta_blk = b;
+    return QTB_OK;
 }
 
 constexpr long long kExtPartBytes = 64LL << 20;  // record rows of ext.cu per launch
@@ -615,6 +638,7 @@ int run_steps(qtb_ctx *c, int j0, int count, bool graph)
             ProfMark pm(c, KC_FORCE);
             launch_ext_steps(c->d, m, c->tabf, c->tab, j0 + t, n, (n + obs - 1) / obs, c->st);
         }
+        CUDA_TRY(cudaGetLastError());
         if (!m.ext_long) return QTB_OK;
     }
     for (int t = 0; t < count; ++t) {
@@ -647,6 +671,7 @@ int run_steps(qtb_ctx *c, int j0, int count, bool graph)
         }
         c->capturing = keep;
     }
+    CUDA_TRY(cudaGetLastError());
     return QTB_OK;
 }
 
@@ -655,21 +680,23 @@ int capture_block(qtb_ctx *c, cudaGraph_t *g)
     CUDA_TRY(cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
     c->capturing = true;
     c->ev_used = 0;
-    int rc;
+    int rc = QTB_OK;
     if (c->gen == QTB_GEN_FOURIER) {
         // a new segment at the first block of each segment (the kernel tests the block clock)
         ProfMark m(c, KC_FILTER);
         launch_fourier(c->d, c->mixed ? 0 : 1, c->max_dofp, c->d.nsys, c->d_sq, c->d_tw,
                        kBlockSteps * c->seg_blocks, 0, c->st);
     } else {
-        { ProfMark m(c, KC_WHITE); gen_white(c, LLONG_MIN); }  // block clock + Kb
-        { ProfMark m(c, KC_FILTER); filter_block(c); }
+        { ProfMark m(c, KC_WHITE); rc = gen_white(c, LLONG_MIN); }  // block clock + Kb
+        if (!rc) { ProfMark m(c, KC_FILTER); rc = filter_block(c); }
     }
-    rc = run_steps(c, 0, kBlockSteps, true);
+    if (!rc) rc = run_steps(c, 0, kBlockSteps, true);
     launch_tick(c->d, c->st);
     c->capturing = false;
     c->ev_pairs = c->ev_used / 2;
     cudaError_t e = cudaStreamEndCapture(c->st, g);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if ((rc || e != cudaSuccess) && *g) cudaGraphDestroy(*g);
     if (rc) return rc;
     if (e != cudaSuccess) return fail(QTB_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
     return QTB_OK;
@@ -1530,15 +1557,17 @@ int qtb_set_filter(qtb_ctx *c, int sys, int mode, int n_taps, double omega_max)
 static int ensure_fresh(qtb_ctx *c)
 {
     if (!c->stale) return QTB_OK;
-    c->stale = false;
-    return refresh_forces(c);
+    const int rc = refresh_forces(c);
+    c->stale = rc != QTB_OK;
+    if (rc) {
+        c->dclock = -1;
+        c->lists_built = false;
+    }
+    return rc;
 }
 
-int qtb_step_n(qtb_ctx *c, long long n)
+static int step_n(qtb_ctx *c, long long n)
 {
-    if (!c) return fail(QTB_ERR_ARG, "null context");
-    if (n < 0) return fail(QTB_ERR_ARG, "n_steps < 0");
-    if (int rc = ensure_fresh(c)) return rc;
     while (n > 0) {
         const long long b = floor_div(c->step, kBlockSteps);
         const int j = (int)(c->step - b * kBlockSteps);
@@ -1546,11 +1575,12 @@ int qtb_step_n(qtb_ctx *c, long long n)
             // the graph generates white block b + Kb and filters block b (filter), or
             // generates a new segment when b starts one (Fourier segments)
             if (c->gen == QTB_GEN_FOURIER) {
-                if (b % c->seg_blocks != 0) ensure_eta(c, b);  // the segment b lies in
+                // the segment b lies in
+                if (int rc = b % c->seg_blocks != 0 ? ensure_eta(c, b) : QTB_OK) return rc;
             } else {
-                ensure_ring(c, b - c->d.Kb, b + c->d.Kb - 1);
+                if (int rc = ensure_ring(c, b - c->d.Kb, b + c->d.Kb - 1)) return rc;
             }
-            set_clock(c, b);
+            if (int rc = set_clock(c, b)) return rc;
             if (c->graph_dirty || !c->gexec) {
                 int rc = build_graph(c);
                 if (rc) return rc;
@@ -1566,7 +1596,7 @@ int qtb_step_n(qtb_ctx *c, long long n)
             n -= kBlockSteps;
             continue;
         }
-        ensure_eta(c, b);
+        if (int rc = ensure_eta(c, b)) return rc;
         const long long mcount = std::min<long long>(n, kBlockSteps - j);
         int rc = run_steps(c, j, (int)mcount, false);
         if (rc) return rc;
@@ -1578,8 +1608,17 @@ int qtb_step_n(qtb_ctx *c, long long n)
         }
         CUDA_TRY(cudaGetLastError());
     }
-    CUDA_TRY(cudaGetLastError());
     return QTB_OK;
+}
+
+int qtb_step_n(qtb_ctx *c, long long n)
+{
+    if (!c) return fail(QTB_ERR_ARG, "null context");
+    if (n < 0) return fail(QTB_ERR_ARG, "n_steps < 0");
+    if (int rc = ensure_fresh(c)) return rc;
+    const int rc = step_n(c, n);
+    if (rc) forget_noise(c);
+    return rc;
 }
 
 int qtb_set_generator(qtb_ctx *c, int generator, int segment_blocks)
@@ -1704,8 +1743,10 @@ int qtb_get_noise(qtb_ctx *c, int sys, double *out, long long *block_out)
     if (!c || !out) return fail(QTB_ERR_ARG, "null argument");
     if (sys < 0 || sys >= (int)c->hs.size()) return fail(QTB_ERR_ARG, "system %d out of range", sys);
     const long long b = floor_div(c->step, kBlockSteps);
-    ensure_eta(c, b);
-    CUDA_TRY(cudaGetLastError());
+    if (int rc = ensure_eta(c, b)) {
+        forget_noise(c);
+        return rc;
+    }
     const DSys &S = c->ds[sys];
     const int D = 3 * S.N * S.P;
     // rows of block b in the noise buffer (Fourier segments hold seg_blocks blocks)

@@ -112,6 +112,7 @@ struct qtb_ctx {
     int taps_cap = 0;
     cudaGraphExec_t gexec = nullptr;
     bool graph_dirty = true;
+    bool filters_ok = false;       // the last set-up of the filters went through
     bool own_stream = false;
     // profiling (events recorded inside the captured block)
     bool profiling = false, capturing = false;
@@ -137,6 +138,7 @@ struct qtb_ctx {
         if (p.dev_alloc) {
             ptr = p.dev_alloc(bytes, p.alloc_user);
         } else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
+            (void)cudaGetLastError();  // the caller reports it (or does without)
             ptr = nullptr;
         }
         if (ptr) allocs.push_back(ptr);
@@ -504,6 +506,7 @@ int setup_tc(qtb_ctx *c)
     const size_t need = (size_t)ns * 256 * Ktot * 2;
     if (need > c->Bt_bytes) {
         c->release(c->d_Bt);
+        c->Bt_bytes = 0;
         c->d_Bt = c->alloc(need);
         if (!c->d_Bt) return fail(QTB_ERR_OOM, "Toeplitz band allocation failed");
         c->Bt_bytes = need;
@@ -732,17 +735,21 @@ int ensure_kappa(qtb_ctx *c, int P)
     double *b = (double *)c->alloc(sizeof(double) * rows);
     double *M = (double *)c->alloc(sizeof(double) * (size_t)n * n);
     double *work = (double *)c->alloc(sizeof(double) * (size_t)(rows + n));
-    if (!F || !A || !b || !M || !work) return fail(QTB_ERR_OOM, "kappa_P solve: device allocation failed");
-    launch_kappa_solve(P, n, ymax, y0, A, b, M, F, work, c->d.err, c->st);
-    CUDA_TRY(cudaGetLastError());
-    int rc = check_err_word(c);
+    int rc = QTB_OK;
+    if (!F || !A || !b || !M || !work) {
+        rc = fail(QTB_ERR_OOM, "kappa_P solve: device allocation failed");
+    } else {
+        launch_kappa_solve(P, n, ymax, y0, A, b, M, F, work, c->d.err, c->st);
+        const cudaError_t e = cudaGetLastError();
+        rc = e != cudaSuccess ? fail(QTB_ERR_CUDA, "kappa_P solve: %s", cudaGetErrorString(e)) : check_err_word(c);
+    }
     c->release(A);
     c->release(b);
     c->release(M);
     c->release(work);
-    if (rc) return rc;
-    c->kappaF[P] = F;
-    return QTB_OK;
+    if (rc) c->release(F);
+    else c->kappaF[P] = F;
+    return rc;
 }
 
 // Fourier-segment generator: sqrt(S_j/n) of every system on the segment grid
@@ -785,8 +792,8 @@ int setup_fourier(qtb_ctx *c, const std::vector<DSpec> &spec)
 constexpr int kFftMinK = 40;
 constexpr size_t kFftMaxRing = (size_t)16 << 30;
 
-// (re)build taps of every system from hs[].mode/n_taps/omega_max
-int rebuild_filters(qtb_ctx *c)
+// (re)build taps of every system from hs[].mode/n_taps/omega_max (rebuild_filters calls it)
+int set_up_filters(qtb_ctx *c)
 {
     const int ns = (int)c->hs.size();
     int tot = 0, Kmax = 0;
@@ -830,6 +837,7 @@ int rebuild_filters(qtb_ctx *c)
         c->release(c->d_taps64);
         c->release(c->d_taps32);
         c->release(c->dS);
+        c->taps_cap = 0;
         c->d_taps64 = (double *)c->alloc(sizeof(double) * tot);
         c->d_taps32 = (float *)c->alloc(sizeof(float) * tot);
         c->dS = (double *)c->alloc(sizeof(double) * 2 * tot);  // spectra, then the cosine tables
@@ -894,6 +902,7 @@ int rebuild_filters(qtb_ctx *c)
         const size_t tb = esz * fft_table_values(nslots, ns);
         if (tb > c->fft_bytes) {
             c->release(c->d_fft);
+            c->fft_bytes = 0;
             c->d_fft = c->alloc(tb);
             if (!c->d_fft) return fail(QTB_ERR_OOM, "filter spectra allocation failed");
             c->fft_bytes = tb;
@@ -912,10 +921,40 @@ int rebuild_filters(qtb_ctx *c)
         int rc = setup_fourier(c, spec);
         if (rc) return rc;
     }
-    c->eta_blk = LLONG_MIN;
-    c->eta_seg = LLONG_MIN;
-    c->graph_dirty = true;
     return QTB_OK;
+}
+
+// set_up_filters replaces buffers as it goes, so from its first line on the captured block
+// and the noise are void, and after a failure the context refuses to step until a later
+// set-up goes through (filters_usable)
+int rebuild_filters(qtb_ctx *c)
+{
+    c->filters_ok = false;
+    c->graph_dirty = true;
+    c->eta_blk = c->eta_seg = LLONG_MIN;
+    const int rc = set_up_filters(c);
+    if (rc) c->ring_hi = c->ring_lo = LLONG_MIN;
+    c->filters_ok = rc == QTB_OK;
+    return rc;
+}
+
+// The same after a change of settings that `undo` takes back: when the new ones cannot be
+// set up, the old ones are, and the failure is the new ones'.
+template <class F> int rebuild_filters_or(qtb_ctx *c, F undo)
+{
+    const int rc = rebuild_filters(c);
+    if (rc == QTB_OK) return rc;
+    const std::string why = g_err;
+    undo();
+    rebuild_filters(c);
+    g_err = why;
+    return rc;
+}
+
+int filters_usable(const qtb_ctx *c)
+{
+    if (c->filters_ok) return QTB_OK;
+    return fail(QTB_ERR_STATE, "the last set-up of the noise filters failed: set them again");
 }
 
 // skin of system s's neighbour lists: a given skin (> 0) for every system, none
@@ -1544,12 +1583,13 @@ int qtb_set_filter(qtb_ctx *c, int sys, int mode, int n_taps, double omega_max)
         if (mode == QTB_NOISE_QTB && c->hs[s].P != 1)
             return fail(QTB_ERR_ARG, "system %d: QTB needs n_beads = 1 (use QTB_PIMD)", s);
     }
+    const std::vector<HSys> before = c->hs;
     for (int s = (sys < 0 ? 0 : sys); s < (sys < 0 ? ns : sys + 1); ++s) {
         c->hs[s].mode = mode;
         c->hs[s].n_taps = (mode == QTB_NOISE_WHITE) ? 1 : n_taps;
         c->hs[s].omega_max = omega_max;
     }
-    return rebuild_filters(c);
+    return rebuild_filters_or(c, [&] { c->hs = before; });
 }
 
 // one force evaluation (lists rebuilt where needed, record of the current step)
@@ -1615,6 +1655,8 @@ int qtb_step_n(qtb_ctx *c, long long n)
 {
     if (!c) return fail(QTB_ERR_ARG, "null context");
     if (n < 0) return fail(QTB_ERR_ARG, "n_steps < 0");
+    if (n > 0)
+        if (int rc = filters_usable(c)) return rc;
     if (int rc = ensure_fresh(c)) return rc;
     const int rc = step_n(c, n);
     if (rc) forget_noise(c);
@@ -1628,29 +1670,24 @@ int qtb_set_generator(qtb_ctx *c, int generator, int segment_blocks)
     const int M = generator == QTB_GEN_FOURIER ? segment_blocks : 1;
     if (M != 1 && M != 2 && M != 4 && M != 8) return fail(QTB_ERR_ARG, "segment_blocks must be 1, 2, 4 or 8");
     CUDA_TRY(cudaStreamSynchronize(c->st));
-    if (M != c->seg_blocks) {
-        void *eta = c->alloc(c->rsz * (size_t)kBlockSteps * M * (size_t)c->d.Dtot);
-        if (!eta) return fail(QTB_ERR_OOM, "noise segment allocation failed");
-        CUDA_TRY(cudaMemsetAsync(eta, 0, c->rsz * (size_t)kBlockSteps * M * (size_t)c->d.Dtot, c->st));
-        c->release(c->d.eta);
-        c->d.eta = eta;
-    }
     const int old_gen = c->gen, old_m = c->seg_blocks;
+    void *const old_eta = c->d.eta, *eta = old_eta;
+    if (M != old_m) {
+        const size_t bytes = c->rsz * (size_t)kBlockSteps * M * (size_t)c->d.Dtot;
+        eta = c->alloc(bytes);
+        if (!eta) return fail(QTB_ERR_OOM, "noise segment allocation failed");
+        CUDA_TRY(cudaMemsetAsync(eta, 0, bytes, c->st));
+    }
     c->gen = generator;
-    c->seg_blocks = M;
-    c->d.eta_blocks = M;
-    int rc = rebuild_filters(c);
-    if (rc) {
+    c->seg_blocks = c->d.eta_blocks = M;
+    c->d.eta = eta;
+    const int rc = rebuild_filters_or(c, [&] {
         c->gen = old_gen;
         c->seg_blocks = c->d.eta_blocks = old_m;
-        if (old_m != M) {
-            c->release(c->d.eta);
-            c->d.eta = c->alloc(c->rsz * (size_t)kBlockSteps * old_m * (size_t)c->d.Dtot);
-        }
-        rebuild_filters(c);
-        return rc;
-    }
-    return QTB_OK;
+        c->d.eta = old_eta;
+    });
+    if (eta != old_eta) c->release(rc ? eta : old_eta);
+    return rc;
 }
 
 int qtb_sync(qtb_ctx *c)
@@ -1730,6 +1767,7 @@ int qtb_get_taps(qtb_ctx *c, int sys, double *h, int max, int *n_out)
 {
     if (!c || !h || !n_out) return fail(QTB_ERR_ARG, "null argument");
     if (sys < 0 || sys >= (int)c->hs.size()) return fail(QTB_ERR_ARG, "system %d out of range", sys);
+    if (int rc = filters_usable(c)) return rc;
     const DSys &S = c->ds[sys];
     const int n = std::min(max, S.K + 1);
     CUDA_TRY(cudaMemcpyAsync(h, c->d_taps64 + S.taps0, sizeof(double) * n, cudaMemcpyDeviceToHost, c->st));
@@ -1743,6 +1781,7 @@ int qtb_get_noise(qtb_ctx *c, int sys, double *out, long long *block_out)
     if (!c || !out) return fail(QTB_ERR_ARG, "null argument");
     if (sys < 0 || sys >= (int)c->hs.size()) return fail(QTB_ERR_ARG, "system %d out of range", sys);
     const long long b = floor_div(c->step, kBlockSteps);
+    if (int rc = filters_usable(c)) return rc;
     if (int rc = ensure_eta(c, b)) {
         forget_noise(c);
         return rc;

@@ -786,7 +786,7 @@ int setup_fourier(qtb_ctx *c, const std::vector<DSpec> &spec)
 }
 
 // The FP64 filter of a system switches to the fast convolution at this half
-// length, as long as its spectra stay within the limit.  Measured, 32769 dofs, ms per
+// length, as long as the context's ring of spectra stays within the limit.  Measured, 32769 dofs, ms per
 // 256 steps (steps included), direct / fast: K = 16 1.83 / 2.35, 32 2.30 / 2.35,
 // 64 3.23 / 2.35, 128 5.11 / 2.36, 1024 31.3 / 2.71.
 constexpr int kFftMinK = 40;
@@ -851,38 +851,35 @@ int set_up_filters(qtb_ctx *c)
     const int Kb = (Kmax + kBlockSteps - 1) / kBlockSteps;
     const int nslots = 2 * Kb + 1;
     const size_t esz = (c->fk == FK_FP64) ? 8 : (c->fk == FK_FP32 ? 4 : 2);
-    // systems with taps long enough for the fast convolution; its spectra take twice
-    // the ring (a context whose device memory does not hold that filters directly)
     const size_t need256 = esz * (size_t)nslots * (size_t)c->d.Dtot * kBlockSteps;
+    auto grow = [&](void *&ptr, size_t &have, size_t bytes) {
+        if (bytes <= have) return true;
+        c->release(ptr);
+        c->ring_hi = c->ring_lo = LLONG_MIN;  // (the ring, or its table with the number of its slots)
+        have = 0;
+        ptr = c->alloc(bytes);
+        if (ptr) have = bytes;
+        return ptr != nullptr;
+    };
+    // systems with taps long enough for the fast convolution.  Its spectra take twice the
+    // ring, of every dof of the context, and a table: a context in which the ring would pass
+    // the limit, or whose device memory does not hold both, filters directly
     bool fft = false;
     for (int s = 0; s < ns; ++s) {
-        c->ds[s].fft = c->fk == FK_FP64 && c->gen == QTB_GEN_FILTER && c->ds[s].K >= kFftMinK &&
-                       2 * esz * (size_t)(2 * ((c->ds[s].K + kBlockSteps - 1) / kBlockSteps) + 1) * (size_t)c->ds[s].dofp * kBlockSteps <= kFftMaxRing;
+        c->ds[s].fft = c->fk == FK_FP64 && c->gen == QTB_GEN_FILTER && c->ds[s].K >= kFftMinK && 2 * need256 <= kFftMaxRing;
         fft = fft || c->ds[s].fft;
     }
-    int row = fft ? 2 * kBlockSteps : kBlockSteps;
-    if (fft && 2 * need256 > c->ring_bytes) {
+    if (fft && !(grow(c->d.ring, c->ring_bytes, 2 * need256) &&
+                 grow(c->d_fft, c->fft_bytes, esz * fft_table_values(nslots, ns)))) {
         c->release(c->d.ring);
+        c->d.ring = nullptr;
         c->ring_bytes = 0;
-        c->d.ring = c->alloc(2 * need256);
-        if (c->d.ring) {
-            c->ring_bytes = 2 * need256;
-        } else {
-            cudaGetLastError();
-            for (int s = 0; s < ns; ++s) c->ds[s].fft = 0;
-            fft = false;
-            row = kBlockSteps;
-        }
-        c->ring_hi = c->ring_lo = LLONG_MIN;
+        for (int s = 0; s < ns; ++s) c->ds[s].fft = 0;
+        fft = false;
     }
-    if (need256 > c->ring_bytes) {
-        c->release(c->d.ring);
-        c->ring_bytes = 0;
-        c->d.ring = c->alloc(need256);
-        if (!c->d.ring) return fail(QTB_ERR_OOM, "noise ring allocation (%zu bytes) failed", need256);
-        c->ring_bytes = need256;
-        c->ring_hi = c->ring_lo = LLONG_MIN;
-    }
+    if (!grow(c->d.ring, c->ring_bytes, need256))
+        return fail(QTB_ERR_OOM, "noise ring allocation (%zu bytes) failed", need256);
+    const int row = fft ? 2 * kBlockSteps : kBlockSteps;
     // which systems' rows are spectra decides what the ring's blocks hold
     std::vector<char> kind(ns);
     for (int s = 0; s < ns; ++s) kind[s] = (char)c->ds[s].fft;
@@ -899,14 +896,6 @@ int set_up_filters(qtb_ctx *c)
     c->d.tapsR = (c->fk == FK_FP64) ? (const void *)c->d_taps64 : (const void *)c->d_taps32;
     CUDA_TRY(cudaMemcpyAsync((void *)c->d.sys, c->ds.data(), sizeof(DSys) * ns, cudaMemcpyHostToDevice, c->st));
     if (c->fft) {
-        const size_t tb = esz * fft_table_values(nslots, ns);
-        if (tb > c->fft_bytes) {
-            c->release(c->d_fft);
-            c->fft_bytes = 0;
-            c->d_fft = c->alloc(tb);
-            if (!c->d_fft) return fail(QTB_ERR_OOM, "filter spectra allocation failed");
-            c->fft_bytes = tb;
-        }
         c->d.fft_tw = c->d_fft;
         c->d.fft_g = (char *)c->d_fft + esz * fft_table_values(0, ns);
         launch_fft_tables(c->d, c->d_taps64, (void *)c->d.fft_tw, (void *)c->d.fft_g, c->st);

@@ -135,3 +135,25 @@ def test_filter_too_long_changes_nothing(qtb, precision):
         assert _same(_go(qtb, ctx), old)
     finally:
         qtb.qtb_destroy(ctx)
+
+
+@pytest.mark.parametrize("atoms,taps", [((80000, 80000), (2049, 2049)), ((165000, 5), (2049, 81))])
+def test_spectra_limit_is_the_contexts(qtb, monkeypatch, atoms, taps):
+    # two systems within the 16 GiB that a ring of spectra may take but not together, and a
+    # short one beside one that passes it alone: no allocation is larger than the limit
+    mem = Memory(qtb, monkeypatch)
+    sizes = []
+    get, free = mem.cb
+    cb = (qtb.ALLOC_FN(lambda nbytes, user: (sizes.append(nbytes), get(nbytes, user))[1]), free)
+    monkeypatch.setattr(qtb, "_torch_allocator", lambda: cb)
+    sys = [W.oscillators(n, 120.0, 4e-3, x0=0.4, spread=0.1, seed=k)[0] for k, n in enumerate(atoms)]
+    ctx = gpu_ctx(qtb, sys, W.well_potential(), 0.5, precision=0, potential=qtb.POT_HARMONIC, ext={"omega": 0.02},
+                  obs_stride=256, max_records=4)
+    try:
+        for k, n in enumerate(taps):
+            qtb.qtb_set_filter(ctx, k, qtb.NOISE_QTB, n, 0.3)
+        dofs = 3 * sum(atoms)
+        assert 2 * 8 * 9 * 256 * dofs > 16 << 30
+        assert 8 * 9 * 256 * dofs <= max(sizes) <= 16 << 30
+    finally:
+        qtb.qtb_destroy(ctx)

@@ -1167,6 +1167,9 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
                 T.nl2e_rho[t] = hi;
                 // the residual of hi rho = -(log2e + 2.0355273740931033e-17)
                 T.nl2e_lo[t] = rho != 0.0 ? (-std::fma(hi, rho, log2e) - 2.0355273740931033e-17) / rho : 0.0;
+                // pair_poly builds 2^a from the low word of a and the exponent field: a rho of either
+                // sign so small that a at the cutoff leaves them takes the library's exp (variant 0)
+                poly_ok = poly_ok && hi * T.rc > -1073741824.0 && hi * T.rc < 1000.0;
             }
             fit_exp2(kExpN, T.ex2c);
         }

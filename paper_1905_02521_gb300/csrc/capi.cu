@@ -1155,8 +1155,17 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
                 F.cf[k] = (float)cf[k];
                 F.ce[k] = (float)ce[k];
             }
+            for (int k = 0; k < 3; ++k) F.cf_lo[k] = (float)(cf[k] - (double)F.cf[k]);
+            for (int k = 0; k < 2; ++k) F.ce_lo[k] = (float)(ce[k] - (double)F.ce[k]);
         }
-        for (int t = 0; t < NT; ++t) F.nl2e_rho[t] = (float)(-log2e * T.inv_rho[t]);
+        F.fshift_lo = (float)(T.fshift - (double)F.fshift);
+        for (int t = 0; t < NT; ++t) {
+            F.nl2e_rho[t] = (float)(-log2e * T.inv_rho[t]);
+            // (times ln 2, and for an r that is low by 1.2e-8: pair_poly)
+            const double lo = (-log2e * T.inv_rho[t] * (1.0 + 1.2e-8) - (double)F.nl2e_rho[t]) * 0.6931471805599453;
+            F.nl2e_lo[t] = std::isfinite(lo) ? (float)lo : 0.0f;
+            F.qq_lo[t] = (float)(T.qq[t] - (double)F.qq[t]);
+        }
         if (c->pair && !c->mixed) {
             poly_ok = T.alpha >= 0.0 && fit_coulomb(T.alpha, T.rc, kFitN<double>, 5e-16, T.cf, T.ce, T.ce_lo);
             T.r2_us = 2.0 / T.rc2;

@@ -735,7 +735,7 @@ __device__ __forceinline__ double my_sqrt(double x) { return sqrt(x); }
 // Coefficients of one type pair, staged in shared memory by the step kernel
 // (the pair type varies across the lanes of a warp).
 template <class R> struct alignas(8 * sizeof(R)) PairRow {
-    R inv_rho, A_over_rho, C6, qq, A, C, eshift, lo;
+    R inv_rho, A_over_rho, C6, qq, A, C, eshift, lo;  // (pair_poly<float>: C is the low word of qq)
 };
 
 template <int VAR, class R> __device__ __forceinline__ PairRow<R> pair_row(const PairTabT<R> &T, int t)
@@ -743,7 +743,8 @@ template <int VAR, class R> __device__ __forceinline__ PairRow<R> pair_row(const
     PairRow<R> p;
     p.inv_rho = VAR ? T.nl2e_rho[t] : T.inv_rho[t];  // (pair_poly takes the exponent in units of ln 2)
     p.A_over_rho = T.A_over_rho[t]; p.C6 = T.C6[t]; p.qq = T.qq[t];
-    p.A = T.A[t]; p.C = T.C[t]; p.eshift = T.eshift[t]; p.lo = VAR ? T.nl2e_lo[t] : R(0);
+    p.A = T.A[t]; p.C = VAR && sizeof(R) == 4 ? T.qq_lo[t] : T.C[t]; p.eshift = T.eshift[t];
+    p.lo = VAR ? T.nl2e_lo[t] : R(0);
     return p;
 }
 
@@ -807,8 +808,19 @@ __device__ __forceinline__ float rsqrt_ftz(float x)
 // that of the form above (modelled: 6.5e-6 against 8.0e-6 relative L2 on 512-ion MgO,
 // 5.8e-6 against 7.4e-6 on LiH).  The context takes it when the fits are accurate to
 // 1e-8 of the Coulomb term at the cutoff (alpha r_cut up to ~1.75).
+//
+// Recorded steps (rec): fv, the force for the virial, and the energy.  They are sums over
+// all pairs, in which what does not average out adds up (the charge inside the cutoff is
+// far from neutral) while the terms largely cancel.  So both get the low words of the
+// constants, of 1/rho and of 1/r (low by 1.4e-8 on average after its Newton step; the exponent
+// takes the 1.2e-8 of the nearest pairs), and what ex2.approx is low by on average (5.0e-8,
+// measured on exponents in [-10, 0]).  Largest error against 64 bits at the edge as its
+// unit is rounded, MgO and LiH of 216 to 1000 ions, relative: V 3.4e-8 and the virial's trace
+// 2.6e-7; without the low words 1.5e-7 and 1.6e-6; the form above 1.4e-7 and 1.4e-6.  RMS
+// of a pair's energy on MgO, modelled: 2.8e-7 eV, 5.4e-7 and 3.9e-7.
+constexpr float kEx2Low = 5.0e-8f;
 __device__ __forceinline__ void pair_poly(const PairTabT<float> &T, const PairRow<float> &P2, float r2, float &f_over_r,
-                                          float &e, bool energy)
+                                          float &fv, float &e, bool rec, bool energy)
 {
     const float y = rsqrt_ftz(r2), t = y * y;
     const float rinv = y * fmaf(-0.5f * r2, t, 1.5f), r2i = fmaf(t, fmaf(-r2, t, 1.0f), t);
@@ -823,14 +835,21 @@ __device__ __forceinline__ void pair_poly(const PairTabT<float> &T, const PairRo
     float ex = ex2_ftz(a);
     ex = fmaf(ex * 0.69314718f, fmaf(r, P2.inv_rho, -a), ex);
     f_over_r = fmaf(P2.qq, p, fmaf(P2.A_over_rho * ex, rinv, -(P2.C6 * r8i)));
-    if (energy) {
-        float q = T.ce[kFitN<float> - 1];
+    fv = e = 0.0f;
+    if (rec) {
+        const float dx = fmaf(r, P2.lo, kEx2Low);  // relative, of ex
+        const float re = fmaf(r2, rinv, -r), rl = (0.5f * rinv) * fmaf(-re, rinv, fmaf(-r, rinv, 1.0f));
+        const float pl = fmaf(r2i, rl, fmaf(-T.fshift_lo, rinv, fmaf(fmaf(T.cf_lo[2], u, T.cf_lo[1]), u, T.cf_lo[0])));
+        fv = f_over_r + fmaf(P2.qq, pl, fmaf(P2.C, p, ((P2.A_over_rho * ex) * rinv) * dx));
+        if (energy) {
+            float q = T.ce[kFitN<float> - 1];
 #pragma unroll
-        for (int k = kFitN<float> - 2; k >= 0; --k) q = fmaf(q, u, T.ce[k]);
-        const float ec = (rinv - q) + fmaf(T.fshift, r - T.rc, -T.erfc_rc_over_rc);
-        e = fmaf(P2.qq, ec, fmaf(P2.A, ex, fmaf(-P2.C, r4i * r2i, -P2.eshift)));
-    } else {
-        e = 0.0f;
+            for (int k = kFitN<float> - 2; k >= 1; --k) q = fmaf(q, u, T.ce[k]);
+            // 1/r - alpha erf(x)/x: two terms of one size, so with their low words too
+            const float ec = fmaf(-u, q, rinv - T.ce[0]) +
+                             ((rl - fmaf(u, T.ce_lo[1], T.ce_lo[0])) + fmaf(T.fshift, r - T.rc, -T.erfc_rc_over_rc));
+            e = fmaf(P2.qq, ec, fmaf(P2.A, fmaf(ex, dx, ex), fmaf(P2.C, ec, fmaf(-P2.C6, (r4i * r2i) * 0.16666667f, -P2.eshift))));
+        }
     }
 }
 
@@ -845,7 +864,7 @@ __device__ __forceinline__ void pair_poly(const PairTabT<float> &T, const PairRo
 // 1.0e-16 instead of 1.8e-16): 1/r^2 rounds once from the exact y^2, the fits are made in
 // double-double.
 __device__ __forceinline__ void pair_poly(const PairTabT<double> &T, const PairRow<double> &P2, double r2,
-                                          double &f_over_r, double &e, bool energy)
+                                          double &f_over_r, double &fv, double &e, bool, bool energy)
 {
     const double y = (double)rsqrt_ftz((float)r2), t = y * y;  // (exact: 24 bits squared)
     const double d = fma(-r2, t, 1.0);
@@ -865,7 +884,7 @@ __device__ __forceinline__ void pair_poly(const PairTabT<double> &T, const PairR
 #pragma unroll
     for (int k = kExpN - 2; k >= 0; --k) ex = fma(ex, f, T.ex2c[k]);
     ex = __hiloint2double(__double2hiint(ex) + (n << 20), __double2loint(ex));
-    f_over_r = fma(P2.qq, p, fma(P2.A_over_rho * ex, rinv, -(P2.C6 * (r4i * r4i))));
+    f_over_r = fv = fma(P2.qq, p, fma(P2.A_over_rho * ex, rinv, -(P2.C6 * (r4i * r4i))));
     if (energy) {
         double q = T.ce[kFitN<double> - 1];
 #pragma unroll
@@ -1152,6 +1171,9 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
     const long long step = d.clock[0] * kBlockSteps + j + 1;
     // (isothermal-isobaric runs reduce K and the virial every step: the cell needs them)
     const bool rec = REC && ((kick == 0) || (step % d.obs_stride == 0) || d.npt != nullptr);
+    // (a cell needs the trace of the virial only: energy and off-diagonal sums where they can
+    // be read, on recorded steps and, without ADV, on the last of a call)
+    const bool erg = rec && !(ADV && d.npt != nullptr && step % d.obs_stride != 0);
     const DSys &S = d.sys[RP.sys];
     const size_t G = (size_t)d.G;
     const long long gi = RP.g0 + (act ? i : 0);
@@ -1217,16 +1239,23 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
     // force (and on recorded steps energy and virial) of one entry, masked by `in`,
     // added to the round's partial sums (px, py, pz)
     auto force = [&](const Geo &g, bool in, R &px, R &py, R &pz) {
-        R fo, ee;
-        if constexpr (VAR) pair_poly(T, ptab[ti * kMaxTypes + g.tj], g.r2, fo, ee, REC && rec);
-        else pair_eval(T, ptab[ti * kMaxTypes + g.tj], g.r2, fo, ee, REC && rec);
+        R fo, fv, ee;
+        if constexpr (VAR) {
+            pair_poly(T, ptab[ti * kMaxTypes + g.tj], g.r2, fo, fv, ee, REC && rec, REC && erg);
+        } else {
+            pair_eval(T, ptab[ti * kMaxTypes + g.tj], g.r2, fo, ee, REC && erg);
+            fv = fo;
+        }
         fo = in ? fo : R(0);
         // stored displacement is r_j - r_i: the force on i is -fo (r_j - r_i)
         px = fma(-fo, g.dx, px); py = fma(-fo, g.dy, py); pz = fma(-fo, g.dz, pz);
         if (REC && rec) {
-            en += in ? ee : R(0);
-            w0 = fma(fo * g.dx, g.dx, w0); w1 = fma(fo * g.dy, g.dy, w1); w2 = fma(fo * g.dz, g.dz, w2);
-            w3 = fma(fo * g.dx, g.dy, w3); w4 = fma(fo * g.dx, g.dz, w4); w5 = fma(fo * g.dy, g.dz, w5);
+            fv = in ? fv : R(0);
+            w0 = fma(fv * g.dx, g.dx, w0); w1 = fma(fv * g.dy, g.dy, w1); w2 = fma(fv * g.dz, g.dz, w2);
+            if (erg) {
+                en += in ? ee : R(0);
+                w3 = fma(fv * g.dx, g.dy, w3); w4 = fma(fv * g.dx, g.dz, w4); w5 = fma(fv * g.dy, g.dz, w5);
+            }
         }
     };
     // One column of a block (kColNE entries) is a group: its terms are summed in R, the
@@ -1345,9 +1374,11 @@ __device__ __forceinline__ void force_unit(const Dev &d, const PairTabT<R> &T, c
     for (int q = 0; q < kNQ; ++q) acc[q] = 0.0;
     float kc = 0.f, kl = 0.f, mc = 0.f, ml = 0.f;  // float-float (hi, lo)
     if (REC && rec) {
-        en = group_sum<LW>(en);
         w0 = group_sum<LW>(w0); w1 = group_sum<LW>(w1); w2 = group_sum<LW>(w2);
-        w3 = group_sum<LW>(w3); w4 = group_sum<LW>(w4); w5 = group_sum<LW>(w5);
+        if (erg) {
+            en = group_sum<LW>(en);
+            w3 = group_sum<LW>(w3); w4 = group_sum<LW>(w4); w5 = group_sum<LW>(w5);
+        }
         if (!kFF && act && (lane & (LW - 1)) == 0) {
             acc[Q_V] = 0.5 * (double)en;
             acc[Q_VIR + 0] = 0.5 * (double)w0; acc[Q_VIR + 1] = 0.5 * (double)w1;

@@ -152,10 +152,13 @@ template <class R> struct PairTabT {
     R rl2;                            // (r_cut + skin)^2: neighbour-list radius
     R erfc_c[12];
     // polynomial variants of the step kernel (pair_poly): with x = alpha r and u = r^2 r2_us - 1,
-    // the Chebyshev fits (monomials in u) of -alpha^3 (erf x - 2 x e^{-x^2}/sqrt(pi))/x^3 (cf)
-    // and alpha erf(x)/x (ce); nl2e_rho = -log2(e)/rho; 2^f on |f| <= 1/2 (FP64 form)
-    R r2_us, cf[kFitN<R>], ce[kFitN<R>], ce_lo[2];
-    R nl2e_rho[kMaxTypes * kMaxTypes], nl2e_lo[kMaxTypes * kMaxTypes];  // (lo: its rounding error)
+    // the interpolants at the Chebyshev nodes (monomials in u) of
+    // -alpha^3 (erf x - 2 x e^{-x^2}/sqrt(pi))/x^3 (cf) and alpha erf(x)/x (ce);
+    // nl2e_rho = -log2(e)/rho; ex2c: 2^f on |f| <= 1/2 (FP64 form).  *_lo: what the rounding of
+    // a constant dropped
+    R r2_us, cf[kFitN<R>], cf_lo[3], ce[kFitN<R>], ce_lo[2];
+    R nl2e_rho[kMaxTypes * kMaxTypes], nl2e_lo[kMaxTypes * kMaxTypes];
+    R qq_lo[kMaxTypes * kMaxTypes], fshift_lo;  // (FP32 form)
     R ex2c[kExpN];
     R hdt_m[kMaxTypes];               // dt / (2 m mvv2e)
     R ext_k[kMaxTypes];               // HARMONIC: m mvv2e w0^2

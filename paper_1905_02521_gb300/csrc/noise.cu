@@ -463,7 +463,8 @@ __global__ void k_kappa_atv(int n, const double *A, const double *s, double *g)
 // roots (they follow for all rows at once).  Every CTA that needs its factor forms it
 // again, which costs less than a launch in between.  (One warp with a row a lane took 85
 // us a panel.)  A non-positive pivot sets ERR_SOLVE (the solve then continues on a
-// placeholder pivot).
+// placeholder pivot).  A block of at most 8 columns ends after 8: on the smallest grid, of 8
+// nodes, all 32 made a solve slower than the form before (P = 2: 0.27 ms, 0.23 before and now).
 constexpr int kCholThreads = 4 * kCholNb;
 
 // 1/v: two Newton steps from the FP32 value where that is in range, else the quotient
@@ -496,6 +497,7 @@ __device__ __forceinline__ void chol_factor32(int n, int k0, const double *M, Ch
     }
 #pragma unroll
     for (int j = 0; j < kCholNb; ++j) {
+        if (j == 8 && k0 + 8 >= n) break;  // the smallest grids: the rest is the identity (uniform)
         double *col = B.col[j & 1];
         if (mine && g == (j & 3)) col[r] = a[j / 4];
         __syncthreads();
@@ -643,12 +645,19 @@ __global__ void __launch_bounds__(32 * kTrsvWarps) k_kappa_trsv(int n, const dou
                 double l[kCholNb];
 #pragma unroll
                 for (int j = 0; j < kCholNb; ++j) l[j] = (pass == 0 ? j < lane : j > lane) ? D[lane][j] : 0.0;
+                const bool more = n - k0 > 8;  // (8 columns or fewer: the rest is the identity)
                 if (pass == 0) {
 #pragma unroll
-                    for (int j = 0; j < kCholNb; ++j) x = fma(-l[j], __shfl_sync(0xffffffffu, x, j), x);
+                    for (int j = 0; j < kCholNb; ++j) {
+                        if (j == 8 && !more) break;
+                        x = fma(-l[j], __shfl_sync(0xffffffffu, x, j), x);
+                    }
                 } else {
+                    if (more)
 #pragma unroll
-                    for (int j = kCholNb - 1; j >= 0; --j) x = fma(-l[j], __shfl_sync(0xffffffffu, x, j), x);
+                        for (int j = kCholNb - 1; j >= 8; --j) x = fma(-l[j], __shfl_sync(0xffffffffu, x, j), x);
+#pragma unroll
+                    for (int j = 7; j >= 0; --j) x = fma(-l[j], __shfl_sync(0xffffffffu, x, j), x);
                 }
                 if (k0 + lane < n) r[k0 + lane] = x * D[lane][lane];
             }

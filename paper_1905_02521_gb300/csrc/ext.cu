@@ -9,7 +9,7 @@
 // same bits however it is cut into launches.  What is left per step is the coloured
 // noise, read once (fetched a step ahead, and a few more into the L2), instead of three
 // launches that each stream the state.  Measured, 10923 atoms x 8 beads, mixed form,
-// a record every 8 steps: 2.0 us a step (2.8 % of it the records' sums) instead of 32.
+// a record every 8 steps: 1.9 us a step instead of 32.
 //
 // Recorded steps: sums over a thread's beads in float-float (FP64 form: FP64), over
 // the CTA in FP64, into a row per record and CTA; k_ext_records then forms the records.
@@ -43,6 +43,24 @@ template <> struct Sum<double> {
     __device__ double value() const { return s; }
 };
 
+// Sums of eight values over a warp by halving: each exchange leaves a lane with half of its
+// values, so that the sums take 9 FP64 additions instead of the 40 of eight butterflies (a
+// warp's FP64 instruction holds its quarter of the SM for 64 cycles).  2 million one-bead atoms,
+// FP32 form, a record every step: 503 us a step, 815 with butterflies, 689 with a launch for
+// every part of a step; FP64 form 1114, 1423, 1383.  Value q ends on lane 4 q.
+__device__ __forceinline__ double warp_sum8(const double (&w)[8], int lane)
+{
+    double a[4], b[2];
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = (h16 ? w[4 + k] : w[k]) + __shfl_xor_sync(0xffffffffu, h16 ? w[k] : w[4 + k], 16);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) b[k] = (h8 ? a[2 + k] : a[k]) + __shfl_xor_sync(0xffffffffu, h8 ? a[k] : a[2 + k], 8);
+    double s = (h4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h4 ? b[0] : b[1], 4);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    return s + __shfl_xor_sync(0xffffffffu, s, 1);
+}
+
 template <class R> __device__ __forceinline__ R ext_force(const PairTabT<R> &T, R kx, R x, R &e)
 {
     if (T.potential == QTB_POT_HARMONIC) {
@@ -75,6 +93,7 @@ __global__ void __launch_bounds__(kExtThreads) k_ext_steps(Dev d, PairTabT<R> T,
     R *X = reinterpret_cast<R *>(d.x), *V = reinterpret_cast<R *>(d.v), *F = reinterpret_cast<R *>(d.f);
     const int ty = d.typ[S.g0 + (act ? i : 0)];
     const R hdtm = T.hdt_m[ty], kx = T.ext_k[ty];
+    const double m = T.mass[ty], hmv = 0.5 * T.mass_mvv[ty], w2 = S.wP * S.wP;
     const R sig = reinterpret_cast<const R *>(d.osig)[unit.x * kMaxTypes + ty];
     const R c1 = sizeof(R) == 4 ? (R)S.c1_f : (R)S.c1, invP = sizeof(R) == 4 ? (R)S.invP_f : (R)S.invP;
     R cs[P], sw[P], ws[P];
@@ -167,23 +186,20 @@ __global__ void __launch_bounds__(kExtThreads) k_ext_steps(Dev d, PairTabT<R> T,
                 for (int b = 0; b < P; ++b) sc.prod((x[b] - x[0]) - dbar, f[b]);
                 const double vb = sv.value() * S.invP;
                 cv = sc.value();
-                k0 = 0.5 * T.mass_mvv[ty] * P * vb * vb;
+                k0 = hmv * P * vb * vb;
             }
-            const double mv = act ? 1.0 : 0.0;
-            const double w[7] = {0.5 * T.mass_mvv[ty] * sK.value() * mv, sV.value() * mv, sX.value() * mv,
-                                 T.mass[ty] * sM.value() * mv, sF.value() * mv, cv * mv, k0 * mv};
-            const double sp = P > 1 ? 0.5 * T.mass_mvv[ty] * S.wP * S.wP * sS.value() * mv : 0.0;
-            double t[8];
+            double w[8] = {hmv * sK.value(), sV.value(), sX.value(), m * sM.value(), sF.value(), cv, k0,
+                           P > 1 ? hmv * w2 * sS.value() : 0.0};
 #pragma unroll
-            for (int u = 0; u < 7; ++u) t[u] = warp_sum(w[u]);
-            t[7] = warp_sum(sp);
+            for (int u = 0; u < 8; ++u) w[u] = act ? w[u] : 0.0;
+            const double t = warp_sum8(w, lane);
             __syncthreads();  // the previous record's row is written
-            if (lane == 0) {
-#pragma unroll
-                for (int u = 0; u < E_N; ++u) red[c][u] = 0.0;
-                red[c][E_K] = t[0]; red[c][E_V] = t[1]; red[c][E_X2] = t[2];
-                red[c][E_MOM + c] = t[3]; red[c][E_VIR + c] = t[4];
-                red[c][E_CV] = t[5]; red[c][E_K0] = t[6]; red[c][E_SPRING] = t[7];
+            if (lane < E_N) red[c][lane] = 0.0;
+            __syncwarp();
+            if ((lane & 3) == 0) {
+                const int q = lane >> 2;
+                red[c][q == 0 ? E_K : q == 1 ? E_V : q == 2 ? E_X2 : q == 3 ? E_MOM + c : q == 4 ? E_VIR + c
+                       : q == 5 ? E_CV : q == 6 ? E_K0 : E_SPRING] = t;
             }
             __syncthreads();
             if (threadIdx.x < E_N)

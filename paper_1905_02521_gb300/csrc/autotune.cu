@@ -87,7 +87,13 @@ extern "C" int qtb_autotune(const qtb_system *sys_in, int n_sys, const qtb_param
     bool beads = false;
     for (int s = 0; s < n_sys; ++s) beads |= sys_in[s].n_beads > 1;
     const double skins[] = {0.5, 0.8, 1.2, 1.6};
-    const int lanes[] = {8, 16, 32};
+    // lanes: by size (up to 128), and the two of the others that are nearest to it.  (An
+    // isothermal-isobaric run records every step, with 16 lanes whatever is asked for.)
+    const int by_size = qtb::lanes_by_size(sys_in, n_sys, p);
+    std::vector<int> lanes = {0};
+    if (!p->npt)
+        for (int ln : {32, 16, 8})
+            if (ln != by_size && lanes.size() < 3) lanes.push_back(ln);
     const int layouts[] = {1, 2};
     const int n_scope = n_sys > 1 ? 2 : 1;
     double best_ms = -1.0;

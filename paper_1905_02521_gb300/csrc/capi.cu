@@ -1040,6 +1040,20 @@ int validate(const qtb_system *sys, int n_sys, const qtb_params *p)
 
 }  // namespace
 
+int qtb::lanes_by_size(const qtb_system *sys, int n_sys, const qtb_params *p)
+{
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    long long n = 0;
+    bool one_bead = true;
+    for (int s = 0; s < n_sys; ++s) {
+        n += (long long)sys[s].n_atoms * sys[s].n_beads;
+        one_bead = one_bead && sys[s].n_beads == 1;
+    }
+    return default_lanes(n, p->precision != QTB_MIXED, one_bead, nsm);
+}
+
 // ===========================================================================
 
 extern "C" {
@@ -1211,12 +1225,8 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
     const double dens_margin = p->npt ? 1.0 / (kCellMinScale * kCellMinScale * kCellMinScale) : 1.0;
     long long beads_total = 0;
     for (int s = 0; s < n_sys; ++s) beads_total += (long long)sys[s].n_atoms * sys[s].n_beads;
-    int dev = 0, nsm = 0;
-    bool one_bead = true;
-    for (int s = 0; s < n_sys; ++s) one_bead = one_bead && sys[s].n_beads == 1;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return bail(fail(QTB_ERR_CUDA, "no CUDA device"));
-    const int lanes = p->list_lanes ? p->list_lanes : default_lanes(beads_total, !c->mixed, one_bead, nsm);
+    const int lanes = p->list_lanes ? p->list_lanes : lanes_by_size(sys, n_sys, p);
+    if (lanes <= 0) return bail(fail(QTB_ERR_CUDA, "no CUDA device"));
     int stage_cap = 0, maxnb = 32;
     if (c->pair) {
         double ecell = 0.0;

@@ -36,6 +36,8 @@ template <class F> cudaError_t allow_dynamic_smem(F kernel, size_t need)
 
 // capi.cu: record the message returned by qtb_last_error(); returns code
 int set_last_error(int code, const char *msg);
+// capi.cu: lanes per bead-atom of the step kernel with qtb_params::list_lanes = 0 (no device: 0)
+int lanes_by_size(const qtb_system *sys, int n_sys, const qtb_params *p);
 
 // mlp.cu: learned kappa_P model (device weights, solver-judged acceptance per P)
 const float *kappa_model_weights(const qtb_kappa_model *M);

@@ -185,7 +185,9 @@ int qtb_init(qtb_ctx **out, const qtb_system *sys, int n_sys, const qtb_params *
  * (Eq. 10, solved in FP64 on the GPU) on w_j = 2 pi j/(L dt), then the taps by
  * an FP64 cosine transform.  Takes effect from the next step; the stochastic
  * trajectory for a given seed does not depend on when it is called, only on
- * the filter in force at each step. */
+ * the filter in force at each step.  On an error the former filters stay in
+ * force; should device memory not hold even those again, the context refuses to
+ * step (QTB_ERR_STATE) until a call of this or qtb_set_generator goes through. */
 int qtb_set_filter(qtb_ctx *c, int sys, int mode, int n_taps, double omega_max);
 
 /* Generator of the coloured noise, for every system of the context.
@@ -200,7 +202,8 @@ int qtb_set_filter(qtb_ctx *c, int sys, int mode, int n_taps, double omega_max);
  *                   mode and cutoff of qtb_set_filter (n_taps unused).  The noise
  *                   is periodic within a segment and uncorrelated across segments.
  * The learned kappa_P mode is not available with QTB_GEN_FOURIER (QTB_ERR_ARG).
- * Takes effect from the next step. */
+ * Takes effect from the next step; on an error the former generator stays, as
+ * with qtb_set_filter. */
 typedef enum { QTB_GEN_FILTER = 0, QTB_GEN_FOURIER = 1 } qtb_generator;
 int qtb_set_generator(qtb_ctx *c, int generator, int segment_blocks);
 
@@ -314,7 +317,8 @@ typedef struct {
 
 /* Autotuner of the launch shapes and the cell/neighbour-list batching.  For
  * every candidate -- skin in {0.5, 0.8, 1.2, 1.6} A (those below r_cut/2),
- * lanes per bead-atom in {8, 16, 32}, for systems with beads the integrator
+ * lanes per bead-atom by size and the two of {8, 16, 32} nearest to that (by
+ * size only at constant pressure), for systems with beads the integrator
  * layouts {1, 2}, and for several systems the rebuild scopes {0, 1} -- it creates a context for the given systems and parameters
  * (qtb_init), applies the filter (noise_mode, n_taps, omega_max; as
  * qtb_set_filter on every system), runs n_blocks 256-step warm-up blocks and

@@ -1,7 +1,7 @@
 // md_kernels.cuh -- device code of the MD hot path (sm_103a) shared by the
-// integrators (md_integrate.cuh, md.cu) and the step kernel (md_step8.cu,
-// md_step16.cu and md_step32.cu: 8, 16 and 32 lanes per bead-atom, compiled in
-// parallel): position representations, reductions, the grid barrier, the mode
+// integrators (md_integrate.cuh, md.cu), the runs in external potentials (ext.cu)
+// and the step kernel (md_step8.cu, md_step16.cu, md_step32.cu and md_step128.cu:
+// 8 to 128 lanes per bead-atom, compiled in parallel): position representations, reductions, the grid barrier, the mode
 // propagator, the list rebuild, the pair force and the step kernel itself.
 //
 // Eq. 4: every bead feels -(1/P) grad V of its own replica plus the ring
@@ -153,7 +153,7 @@ struct DD {
     __device__ double value() const { return hi; }
 };
 
-// Sums of x, y and z over an aligned group of W lanes (8, 16 or 32), by halving: the
+// Sums of x, y and z over an aligned group of W lanes (8 or 16), by halving: the
 // first exchange leaves a lane with x and y or with z, the second with one of them,
 // the rest add up that component.  Five float-float additions instead of twelve (the
 // reductions were a seventh of the step kernel's instructions at 16 lanes), each sum

@@ -202,7 +202,7 @@ struct Dev {
     int *cnt;             // [ncells] running counts (binning)
     int *ccount;          // [ncells] counts after sorting
     int *cidx;            // [ncells * cap] bead-atom index, sorted
-    void *cpos;           // [ncells * cap] packed {x, y, z, replica-local index} (int4 or 4 doubles)
+    void *cpos;           // [ncells * cap] packed {x, y, z, type} (int4 or 4 doubles)
     // neighbour lists (pair potential)
     // packed positions {x, y, z, type} (int4 or 4 doubles), [G] in slot order (replica
     // by replica, in the order of the cells of the last rebuild, so that the gathers of
